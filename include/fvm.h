@@ -320,7 +320,7 @@ fvm_status fvm_projection_vjp(fvm_case* c, double dt, const double* host_ybar, d
    The results are those of stepping each case alone (tested bitwise).
 
    Requirements: every case has the same precision, runs the default
-   one-sweep level kernels and the single-CTA coarse levels, and has
+   one-sweep level kernels and the cluster-cycled coarse levels, and has
    profiling off.  While a case belongs to a live batch, step it only
    through the batch.  Memory: the batch holds device tables of its launch
    arguments (kilobytes per case) per pointer parity; the cases keep their

@@ -192,19 +192,26 @@ struct SolveState {
     double g_dq;             // (d, A d) of the kept direction
 };
 
-// Levels lc..L-1, cycled by one CTA in shared memory.
 // per-sweep Jacobi weights of the Chebyshev smoother (smoother 1: at most this many sweeps a side)
 constexpr int kMaxChebSweeps = 16;
 
-struct CoarseLevels {
-    int32_t nl;              // number of levels handled
+// How a cluster of S blocks cycles the levels lc .. (coarse_kernels.cu): each level's planes
+// along its outermost active axis (ns planes of P cells, m to a block) and its arrays in the
+// blocks' shared memory.  The same layout in every block.
+struct CoarsePlan {
+    int32_t S, lc, nl;
+    int32_t lm;              // the first lm levels are dealt out over the blocks, block 0 keeps the rest
     int32_t pre, post;
     int32_t cheb;            // 1: sweep i of a side takes w[side][i] (0 pre, 1 post); 0: the level's wJ
-    LevelDev lv[FVM_MAX_LEVELS];
+    int32_t dense_all, x;
+    size_t smem;
+    struct Level {
+        LevelDev dev;
+        int32_t slow, P, ns, m, e0, e1, r, f;
+        uint32_t dir;
+    } lv[FVM_MAX_LEVELS];
     double w[2][kMaxChebSweeps];
-    float wf[2][kMaxChebSweeps];
 };
-
 
 // ---------------------------------------------------------------- helpers
 __host__ __device__ __forceinline__ int64_t cell_index(int i, int j, int k, int nx, int ny) {
@@ -244,6 +251,59 @@ template <> struct LP<float> {
     static __device__ __forceinline__ float diag(const LevelDev& L) { return L.diagf; }
     static __device__ __forceinline__ float ih2a(const LevelDev& L, int a) { return L.ih2af[a]; }
 };
+
+// ---------------------------------------------------------------- prolongation
+// Trilinear prolongation of a coarse field at fine cell (i,j,k) (Eq.
+// prolongation): per active axis 3/4 of the parent and 1/4 of the parent's
+// neighbour on the fine cell's side.  A neighbour beyond a domain face is the
+// coarse level's ghost of the clamped cell (the boundary rules of Section 2.7
+// on every level): the cell's own value across a zero-gradient face, its
+// negative across a zero-value (outlet) face; at an edge or corner the signs
+// of both faces apply.  get(q) reads the coarse value, code(q) the coarse
+// cell's 16-bit neighbour code (two bits per face, 2 = zero-value).
+template <class C, class G, class F>
+__device__ __forceinline__ C prolong_at(const int* fa, const int* cn, int i, int j, int k, G get, F code) {
+    const int f[3] = {i, j, k};
+    int P[3], Q[3], side[3];
+    bool out[3];
+    C w[3][2];
+    for (int a = 0; a < 3; ++a) {
+        out[a] = false;
+        side[a] = 0;
+        if (fa[a]) {
+            P[a] = f[a] >> 1;
+            const int q = P[a] + ((f[a] & 1) ? 1 : -1);
+            out[a] = q < 0 || q >= cn[a];
+            side[a] = q < 0 ? 0 : 1;
+            Q[a] = out[a] ? P[a] : q;
+            w[a][0] = (C)0.75;
+            w[a][1] = (C)0.25;
+        } else {
+            P[a] = Q[a] = f[a];
+            w[a][0] = (C)1;
+            w[a][1] = (C)0;
+        }
+    }
+    C acc = (C)0;
+    for (int sz = 0; sz < (fa[2] ? 2 : 1); ++sz)
+        for (int sy = 0; sy < (fa[1] ? 2 : 1); ++sy)
+            for (int sx = 0; sx < (fa[0] ? 2 : 1); ++sx) {
+                const int ii = sx ? Q[0] : P[0], jj = sy ? Q[1] : P[1], kk = sz ? Q[2] : P[2];
+                const int q = ii + cn[0] * (jj + cn[1] * kk);
+                C v = get(q);
+                const bool gx = sx && out[0], gy = sy && out[1], gz = sz && out[2];
+                if (gx || gy || gz) {
+                    const uint32_t fc = code(q);
+                    bool neg = false;
+                    if (gx) neg ^= ((fc >> (2 * (0 + side[0]))) & 3u) == 2u;
+                    if (gy) neg ^= ((fc >> (2 * (2 + side[1]))) & 3u) == 2u;
+                    if (gz) neg ^= ((fc >> (2 * (4 + side[2]))) & 3u) == 2u;
+                    if (neg) v = -v;
+                }
+                acc += w[0][sx] * w[1][sy] * w[2][sz] * v;
+            }
+    return acc;
+}
 
 // ---------------------------------------------------------------- launchers
 struct StatePtrs {
@@ -304,7 +364,13 @@ cudaError_t launch_resid_restrict(int inner, const LevelDev& Lf, const LevelDev&
                                   void* rc, void* ec0, const SolveState* st, cudaStream_t s);
 cudaError_t launch_prolong_add(int inner, const LevelDev& Lf, const LevelDev& Lc, const void* ec, void* e,
                                const SolveState* st, cudaStream_t s);
-cudaError_t prepare_coarse_cta(int inner, size_t smem);
+// the cluster's share of the levels: the finest level that a cluster of S blocks takes (S smaller
+// where that leaves nothing to deal out, unless exact), the partition and the layout
+bool coarse_plan(const std::vector<LevelDev>& levels, const std::vector<uint32_t>& dir, int inner, int S, bool exact,
+                 CoarsePlan& pl);
+int coarse_cluster_for(int cases);   // blocks per cluster when this many cases run theirs at once
+// sets the kernel's limits; an error where the device cannot run such a cluster
+cudaError_t prepare_coarse(int inner, const CoarsePlan& pl);
 // flexible CG with one kept direction around the V-cycles: the inner products
 // of z (the V-cycles' correction) with A z, r and the kept direction d_prev
 // (last block: beta, alpha), then d = z - beta d_prev, p += alpha d, d kept.
@@ -321,12 +387,11 @@ cudaError_t launch_prolong_nearest_to_p(int inner, const LevelDev& Lf, const Lev
                                         const SolveState* st, cudaStream_t s);
 cudaError_t launch_jacobi_p(int bprec, const LevelDev& L, double* p, const void* b, double* q, const SolveState* st,
                             cudaStream_t s);
-cudaError_t launch_coarse_cta(int inner, const CoarseLevels& cl, const void* r_in, void* e_out, const double* Ainv,
-                              const SolveState* st, cudaStream_t s);
+cudaError_t launch_coarse(int inner, const CoarsePlan& pl, const void* r_in, void* e_out, const double* Ainv,
+                          const SolveState* st, cudaStream_t s);
 cudaError_t launch_convert(int src_prec, int dst_prec, const void* src, void* dst, int64_t N, cudaStream_t s);
 int resid0_blocks(int nx, int ny, int nz);
 int level0_blocks_max(int nx, int ny, int nz);   // blocks of any level-0 reduction pass, at most
-size_t coarse_cta_smem(const CoarseLevels& cl, int inner);
 // ---------------------------------------------------------------- one case or many per launch
 // Every step and multigrid kernel is a functor K with `static constexpr int
 // kThreads` and `__device__ void run(const BlockAt&) const` (the level-0

@@ -30,7 +30,6 @@ template <class T> struct Acc { using type = T; };
 template <> struct Acc<__nv_bfloat16> { using type = float; };
 
 constexpr int BX = 32, BY = 4, BZ = 2;
-constexpr int kCtaThreads = 1024;
 
 __device__ __forceinline__ bool cell3(const LevelDev& L, const BlockAt& at, int& i, int& j, int& k) {
     i = at.b.x * BX + threadIdx.x;
@@ -320,58 +319,6 @@ __device__ void ResidRestrictK<TI>::run(const BlockAt& at) const {
                 sum += to_c<C>(ldg(r + c)) - apply_A<C>(Lf, f, e, c, eP);
             }
     store_restricted<TI, C>(Lc, rc, ec0, I + Lc.n[0] * (J + Lc.n[1] * K), sum / (C)(fx * fy * fz));
-}
-
-// Trilinear prolongation of a coarse field at fine cell (i,j,k) (Eq.
-// prolongation): per active axis 3/4 of the parent and 1/4 of the parent's
-// neighbour on the fine cell's side.  A neighbour beyond a domain face is the
-// coarse level's ghost of the clamped cell (the boundary rules of Section 2.7
-// on every level): the cell's own value across a zero-gradient face, its
-// negative across a zero-value (outlet) face; at an edge or corner the signs
-// of both faces apply.  get(q) reads the coarse value, code(q) the coarse
-// cell's 16-bit neighbour code (two bits per face, 2 = zero-value).
-template <class C, class G, class F>
-__device__ __forceinline__ C prolong_at(const int* fa, const int* cn, int i, int j, int k, G get, F code) {
-    const int f[3] = {i, j, k};
-    int P[3], Q[3], side[3];
-    bool out[3];
-    C w[3][2];
-    for (int a = 0; a < 3; ++a) {
-        out[a] = false;
-        side[a] = 0;
-        if (fa[a]) {
-            P[a] = f[a] >> 1;
-            const int q = P[a] + ((f[a] & 1) ? 1 : -1);
-            out[a] = q < 0 || q >= cn[a];
-            side[a] = q < 0 ? 0 : 1;
-            Q[a] = out[a] ? P[a] : q;
-            w[a][0] = (C)0.75;
-            w[a][1] = (C)0.25;
-        } else {
-            P[a] = Q[a] = f[a];
-            w[a][0] = (C)1;
-            w[a][1] = (C)0;
-        }
-    }
-    C acc = (C)0;
-    for (int sz = 0; sz < (fa[2] ? 2 : 1); ++sz)
-        for (int sy = 0; sy < (fa[1] ? 2 : 1); ++sy)
-            for (int sx = 0; sx < (fa[0] ? 2 : 1); ++sx) {
-                const int ii = sx ? Q[0] : P[0], jj = sy ? Q[1] : P[1], kk = sz ? Q[2] : P[2];
-                const int q = ii + cn[0] * (jj + cn[1] * kk);
-                C v = get(q);
-                const bool gx = sx && out[0], gy = sy && out[1], gz = sz && out[2];
-                if (gx || gy || gz) {
-                    const uint32_t fc = code(q);
-                    bool neg = false;
-                    if (gx) neg ^= ((fc >> (2 * (0 + side[0]))) & 3u) == 2u;
-                    if (gy) neg ^= ((fc >> (2 * (2 + side[1]))) & 3u) == 2u;
-                    if (gz) neg ^= ((fc >> (2 * (4 + side[2]))) & 3u) == 2u;
-                    if (neg) v = -v;
-                }
-                acc += w[0][sx] * w[1][sy] * w[2][sz] * v;
-            }
-    return acc;
 }
 
 template <class TI>
@@ -1532,279 +1479,6 @@ __device__ void RRWalkK<TI>::run(const BlockAt& at) const {
     }
 }
 
-// ------------------------------------------------------------------ coarse levels in one CTA
-// V-cycle over levels lc..L-1 in shared memory: reads r on level lc from
-// global memory, writes the correction e on level lc.
-// A level's stencil constants in registers for the coarse CTA's cell loops (the level
-// descriptions live in shared memory, which the loops also write, so the compiler would reload
-// them for every cell), and A e with them: a cell whose face codes are all 0 on three active
-// axes takes the six neighbours without the per-face code selects, in the same arithmetic order
-// as apply_A_with, so both forms give the same value
-template <class C>
-struct CtaStencil {
-    int sy, sz;
-    C ih[3];
-    bool act[3];
-    bool all3;
-};
-
-template <class C>
-__device__ __forceinline__ CtaStencil<C> cta_stencil(const LevelDev& L) {
-    CtaStencil<C> S;
-    S.sy = L.n[0];
-    S.sz = L.n[0] * L.n[1];
-    for (int a = 0; a < 3; ++a) {
-        S.ih[a] = LP<C>::ih2(L, a);
-        S.act[a] = L.active[a] != 0;
-    }
-    S.all3 = S.act[0] && S.act[1] && S.act[2];
-    return S;
-}
-
-template <class C>
-__device__ __forceinline__ C cta_A(const CtaStencil<C>& S, uint32_t f, const C* e, int c, C eP) {
-    if (S.all3 && (f & 0xfffu) == 0u) {
-        C acc = ((eP - e[c - 1]) + (eP - e[c + 1])) * S.ih[0];
-        acc += ((eP - e[c - S.sy]) + (eP - e[c + S.sy])) * S.ih[1];
-        acc += ((eP - e[c - S.sz]) + (eP - e[c + S.sz])) * S.ih[2];
-        return acc;
-    }
-    const int st[3] = {1, S.sy, S.sz};
-    C acc = (C)0;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        if (!S.act[a]) continue;
-        const C lo = nb_val<C>((f >> (4 * a)) & 3u, c - st[a], eP, [&](int q) { return e[q]; });
-        const C hi = nb_val<C>((f >> (4 * a + 2)) & 3u, c + st[a], eP, [&](int q) { return e[q]; });
-        acc += ((eP - lo) + (eP - hi)) * S.ih[a];
-    }
-    return acc;
-}
-
-// the weight of sweep i on one side (0 pre, 1 post) of a coarse-CTA level
-template <class C> __device__ __forceinline__ C coarse_weight(const CoarseLevels& cl, const LevelDev& L, int side, int i);
-template <> __device__ __forceinline__ double coarse_weight<double>(const CoarseLevels& cl, const LevelDev& L, int side,
-                                                                   int i) {
-    return cl.cheb ? cl.w[side][i] : L.wJ;
-}
-template <> __device__ __forceinline__ float coarse_weight<float>(const CoarseLevels& cl, const LevelDev& L, int side,
-                                                                 int i) {
-    return cl.cheb ? cl.wf[side][i] : L.wJf;
-}
-
-template <class TI>
-struct CoarseK {
-    static constexpr int kThreads = kCtaThreads;
-    CoarseLevels cl;
-    const TI* r_in;
-    TI* e_out;
-    const double* Ainv;
-    const SolveState* st;
-    __device__ bool live() const { return st->active != 0; }   // batched: skip a converged case
-    __device__ void run(const BlockAt& at) const;
-};
-
-template <class TI>
-__device__ void coarse_cta_body(const CoarseLevels& cl, const TI* __restrict__ r_in, TI* __restrict__ e_out,
-                                const double* __restrict__ Ainv);
-
-template <class TI>
-__device__ void CoarseK<TI>::run(const BlockAt&) const {
-    coarse_cta_body<TI>(cl, r_in, e_out, Ainv);
-}
-
-// c / n for the small levels of the coarse kernel (0 <= c < 2^22, inv_n = 1/n in FP32):
-// (c + 1/2)/n is at least 1/(2n) from an integer, more than the FP32 rounding of the product
-__device__ __forceinline__ int small_div(int c, float inv_n) { return (int)(((float)c + 0.5f) * inv_n); }
-
-template <class TI>
-__device__ void coarse_cta_body(const CoarseLevels& cl, const TI* __restrict__ r_in, TI* __restrict__ e_out,
-                                const double* __restrict__ Ainv) {
-    using C = typename Acc<TI>::type;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    // level descriptions and array bases live in shared memory (one copy per CTA)
-    __shared__ LevelDev lvs[FVM_MAX_LEVELS];
-    // the arrays' offsets into the dynamic shared memory (elements of C, codes in 16-bit units):
-    // pointers formed from smem_raw here let the compiler address them as shared memory (pointers
-    // kept in a shared array would be generic, each access a generic load)
-    __shared__ int E0o[FVM_MAX_LEVELS];
-    __shared__ int E1o[FVM_MAX_LEVELS];
-    __shared__ int Ro[FVM_MAX_LEVELS];
-    __shared__ int Fo[FVM_MAX_LEVELS];
-    C* const Cs = reinterpret_cast<C*>(smem_raw);
-    uint16_t* const Us = reinterpret_cast<uint16_t*>(smem_raw);
-    auto E0 = [&](int l) { return Cs + E0o[l]; };
-    auto E1 = [&](int l) { return Cs + E1o[l]; };
-    auto R = [&](int l) { return Cs + Ro[l]; };
-    auto F = [&](int l) { return Us + Fo[l]; };
-    const int T = blockDim.x, tid = threadIdx.x;
-    // the level descriptions, copied word by word by all threads
-    {
-        const int words = cl.nl * (int)(sizeof(LevelDev) / 4);
-        const uint32_t* src = reinterpret_cast<const uint32_t*>(cl.lv);
-        for (int w = tid; w < words; w += T) reinterpret_cast<uint32_t*>(lvs)[w] = src[w];
-    }
-    if (tid == 0) {
-        int q = 0;
-        for (int l = 0; l < cl.nl; ++l) {
-            const int N = (int)cl.lv[l].N;
-            E0o[l] = q; q += N;
-            E1o[l] = q; q += N;
-            Ro[l] = q; q += N;
-        }
-        int u = q * (int)(sizeof(C) / sizeof(uint16_t));
-        for (int l = 0; l < cl.nl; ++l) {
-            Fo[l] = u;
-            u += (int)cl.lv[l].N;
-        }
-    }
-    __syncthreads();
-    for (int l = 0; l < cl.nl; ++l) {
-        const int N = (int)lvs[l].N;
-        const uint16_t* src = lvs[l].nbf;   // the level's codes in global memory
-        for (int c = tid; c < N; c += T) F(l)[c] = src[c];
-    }
-    {
-        const int N0 = (int)lvs[0].N;
-        for (int c = tid; c < N0; c += T) R(0)[c] = to_c<C>(r_in[c]);
-    }
-    __syncthreads();
-    __shared__ int cur[FVM_MAX_LEVELS];
-    // down: pre-smooth, restrict
-    for (int l = 0; l + 1 < cl.nl; ++l) {
-        const LevelDev& L = lvs[l];
-        const CtaStencil<C> S = cta_stencil<C>(L);
-        const uint16_t* const fl = F(l);
-        C* const rl = R(l);
-        const int N = (int)L.N;
-        const C iD = LP<C>::iD(L);
-        const C w0 = coarse_weight<C>(cl, L, 0, 0);
-        for (int c = tid; c < N; c += T) E0(l)[c] = is_solid(fl[c]) ? (C)0 : w0 * rl[c] * iD;
-        __syncthreads();
-        int s = 0;
-        for (int it = 1; it < cl.pre; ++it) {
-            const C w = coarse_weight<C>(cl, L, 0, it);
-            C* ein = s ? E1(l) : E0(l);
-            C* eo = s ? E0(l) : E1(l);
-            for (int c = tid; c < N; c += T) {
-                const uint32_t f = fl[c];
-                C v = (C)0;
-                if (!is_solid(f)) {
-                    const C eP = ein[c];
-                    v = eP + w * (rl[c] - cta_A<C>(S, f, ein, c, eP)) * iD;
-                }
-                eo[c] = v;
-            }
-            s ^= 1;
-            __syncthreads();
-        }
-        if (tid == 0) cur[l] = s;
-        const LevelDev& Lc = lvs[l + 1];
-        const C* e = s ? E1(l) : E0(l);
-        const int fx = L.active[0] ? 2 : 1, fy = L.active[1] ? 2 : 1, fz = L.active[2] ? 2 : 1;
-        const int Nc = (int)Lc.N, cn0 = Lc.n[0], cn1 = Lc.n[1], n0 = L.n[0], n1 = L.n[1];
-        const float icn0 = 1.0f / (float)cn0, icn01 = 1.0f / (float)(cn0 * cn1);
-        C* const rc = R(l + 1);
-        // one child per thread: eight consecutive lanes hold one coarse cell's children
-        // (missing children of a collapsed axis add 0) and sum them by a fixed shuffle tree
-        const int items = 8 * Nc, bound = (items + 31) & ~31;
-        for (int w = tid; w < bound; w += T) {
-            const int cc = w >> 3, ch = w & 7;
-            const int dx = ch & 1, dy = (ch >> 1) & 1, dz = ch >> 2;
-            C v = (C)0;
-            if (w < items && dx < fx && dy < fy && dz < fz) {
-                const int K = small_div(cc, icn01);
-                const int rem = cc - K * cn0 * cn1;
-                const int J = small_div(rem, icn0);
-                const int I = rem - J * cn0;
-                const int c = (I * fx + dx) + n0 * ((J * fy + dy) + n1 * (K * fz + dz));
-                const uint32_t f = fl[c];
-                if (!is_solid(f)) v = rl[c] - cta_A<C>(S, f, e, c, e[c]);
-            }
-            v += __shfl_xor_sync(0xffffffffu, v, 1);
-            v += __shfl_xor_sync(0xffffffffu, v, 2);
-            v += __shfl_xor_sync(0xffffffffu, v, 4);
-            if (ch == 0 && w < items) rc[cc] = v / (C)(fx * fy * fz);
-        }
-        __syncthreads();
-    }
-    // coarsest: dense solve, one warp per row (coalesced reads of the inverse); in the
-    // reduced-precision modes from the FP32 copy of the inverse stored after the FP64 one
-    {
-        const int l = cl.nl - 1;
-        const int N = (int)lvs[l].N;
-        const int lane = tid & 31, warp = tid >> 5, nw = T >> 5;
-        for (int row = warp; row < N; row += nw) {
-            if constexpr (sizeof(C) == 8) {
-                double acc = 0.0;
-                const double* a = Ainv + (size_t)row * N;
-                for (int col = lane; col < N; col += 32) acc += __ldg(a + col) * (double)R(l)[col];
-                for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-                if (lane == 0) E0(l)[row] = (C)acc;
-            } else {
-                float acc = 0.0f;
-                const float* a = reinterpret_cast<const float*>(Ainv + (size_t)N * N) + (size_t)row * N;
-                for (int col = lane; col < N; col += 32) acc = fmaf(__ldg(a + col), R(l)[col], acc);
-                for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-                if (lane == 0) E0(l)[row] = acc;
-            }
-        }
-        if (tid == 0) cur[l] = 0;
-        __syncthreads();
-    }
-    // up: prolong, post-smooth
-    for (int l = cl.nl - 2; l >= 0; --l) {
-        const LevelDev& L = lvs[l];
-        const LevelDev& Lc = lvs[l + 1];
-        const CtaStencil<C> S = cta_stencil<C>(L);
-        C* const Rl = R(l);
-        const uint16_t* const fl = F(l);
-        const uint16_t* const fc = F(l + 1);
-        // the prolongation's axes and coarse extents in registers (see CtaStencil)
-        const int fa[3] = {L.active[0], L.active[1], L.active[2]};
-        const int cn[3] = {Lc.n[0], Lc.n[1], Lc.n[2]};
-        const int N = (int)L.N, n0 = L.n[0], n1 = L.n[1];
-        const float in0 = 1.0f / (float)n0, in01 = 1.0f / (float)(n0 * n1);
-        const C* ec = cur[l + 1] ? E1(l + 1) : E0(l + 1);
-        C* e = cur[l] ? E1(l) : E0(l);
-        for (int c = tid; c < N; c += T) {
-            if (is_solid(fl[c])) continue;
-            const int k = small_div(c, in01);
-            const int rem = c - k * n0 * n1;
-            const int j = small_div(rem, in0);
-            const int i = rem - j * n0;
-            e[c] += prolong_at<C>(fa, cn, i, j, k, [&](int q) { return ec[q]; },
-                                  [&](int q) { return (uint32_t)fc[q]; });
-        }
-        __syncthreads();
-        int s = cur[l];
-        const C iD = LP<C>::iD(L);
-        for (int it = 0; it < cl.post; ++it) {
-            const C w = coarse_weight<C>(cl, L, 1, it);
-            C* ein = s ? E1(l) : E0(l);
-            C* eo = s ? E0(l) : E1(l);
-            for (int c = tid; c < N; c += T) {
-                const uint32_t f = fl[c];
-                C v = (C)0;
-                if (!is_solid(f)) {
-                    const C eP = ein[c];
-                    v = eP + w * (Rl[c] - cta_A<C>(S, f, ein, c, eP)) * iD;
-                }
-                eo[c] = v;
-            }
-            s ^= 1;
-            __syncthreads();
-        }
-        if (tid == 0) cur[l] = s;
-        __syncthreads();
-    }
-    {
-        const C* e = cur[0] ? E1(0) : E0(0);
-        const int N0 = (int)lvs[0].N;
-        for (int c = tid; c < N0; c += T) e_out[c] = from_c<TI, C>(e[c]);
-    }
-}
-
 // ------------------------------------------------------------------ flexible CG acceleration (krylov = 1)
 // One pass over level 0 with z (the V-cycles' correction for the outer
 // residual r) and the kept direction d_prev: A z at each cell from the
@@ -2062,16 +1736,6 @@ int level0_blocks_max(int nx, int ny, int nz) {
     return most;
 }
 
-size_t coarse_cta_smem(const CoarseLevels& cl, int inner) {
-    const size_t cs = inner == FVM_FP64 ? 8 : 4;
-    size_t n = 0, m = 0;
-    for (int l = 0; l < cl.nl; ++l) {
-        n += 3 * (size_t)cl.lv[l].N;
-        m += (size_t)cl.lv[l].N;
-    }
-    return n * cs + m * 2 + 16;
-}
-
 #define DISPATCH_I(inner, ...)                                            \
     do {                                                                  \
         if ((inner) == FVM_FP64) { using TI = double; __VA_ARGS__; }      \
@@ -2259,23 +1923,6 @@ cudaError_t launch_prolong_add(int inner, const LevelDev& Lf, const LevelDev& Lc
                         grid, dim3(TX, TY), 0, s);
     }
     DISPATCH_I(inner, err = launch_k(ProlongK<TI>{Lf, Lc, (const TI*)ec, (TI*)e, st}, grid3(Lf), kBlock3, 0, s));
-    return err;
-}
-
-cudaError_t prepare_coarse_cta(int inner, size_t smem) {
-    DISPATCH_I(inner, {
-        cudaError_t err = raise_smem_limit((const void*)k_one<CoarseK<TI>>, smem);
-        if (err != cudaSuccess) return err;
-    });
-    return cudaSuccess;
-}
-
-cudaError_t launch_coarse_cta(int inner, const CoarseLevels& cl, const void* r_in, void* e_out, const double* Ainv,
-                              const SolveState* st, cudaStream_t s) {
-    const size_t smem = coarse_cta_smem(cl, inner);
-    cudaError_t err = cudaSuccess;
-    DISPATCH_I(inner, err = launch_k(CoarseK<TI>{cl, (const TI*)r_in, (TI*)e_out, Ainv, st}, dim3(1),
-                                     dim3(kCtaThreads), smem, s));
     return err;
 }
 

@@ -331,12 +331,13 @@ struct fvm_case {
     void* nut = nullptr;             // nu_t of the state after a destruction half step
     bool nut_valid = false;          // nut matches the current k, omega
     std::vector<DevLevel> levels;
+    std::vector<uint32_t> level_dir; // per level: the faces (bits) with a zero-value cell
     SolveState* sst = nullptr;       // device
     SolveState* h_sst = nullptr;     // pinned host copy
-    size_t lc = 0;                   // first level cycled by the single-CTA coarse kernel
     int inner_cycles = 1;            // V-cycles per outer residual (adaptive solves)
     int rule_inner = 1;              // the same for the rule in force (1 for fixed-count solves)
-    CoarseLevels coarse;
+    CoarsePlan coarse;               // the levels cycled by one cluster, stepped alone
+    CoarsePlan coarse_many;          // and in the batch being captured
     // CUDA graphs of whole time steps, keyed by the field pointers they were captured with
     bool use_graph = true;
     struct StepGraph {
@@ -742,10 +743,13 @@ LevelDev weighted(LevelDev v, double w) {
     return v;
 }
 
+// how the coarse levels are cycled in the launches being issued or recorded
+const CoarsePlan& coarse_of(const fvm_case* c) { return g_rec ? c->coarse_many : c->coarse; }
+
 // Level l (> 0) gets its first Jacobi sweep from the restriction that forms its r
-// (not the levels the single-CTA coarse kernel cycles).
+// (not the levels that the cluster kernel cycles).
 bool first_sweep_fused(const fvm_case* c, size_t l) {
-    return l > 0 && l < c->lc;
+    return l > 0 && l < (size_t)coarse_of(c).lc;
 }
 
 // One V-cycle of the correction equation on levels l.. with r on level l;
@@ -760,12 +764,13 @@ fvm_status cycle(fvm_case* c, size_t l, int& out_idx) {
     cudaStream_t s = c->stream;
     const double N = (double)L.dev.N;
     const double si = (double)elem_size(c->inner);
-    if (l == c->lc) {
+    const CoarsePlan& cp = coarse_of(c);
+    if (l == (size_t)cp.lc) {
         const double nco = (double)c->levels.back().dev.N;
         double cells = 0.0;
         for (size_t q = l; q < c->levels.size(); ++q) cells += (double)c->levels[q].dev.N;
         KLAUNCH("coarse_cta", 2 * N * si + nco * nco * 8 + 2 * cells, 1,
-                launch_coarse_cta(c->inner, c->coarse, L.r, L.e[0], c->Ainv, c->sst, s));
+                launch_coarse(c->inner, cp, L.r, L.e[0], c->Ainv, c->sst, s));
         out_idx = 0;
         return FVM_OK;
     }
@@ -1088,6 +1093,23 @@ int field_slot(int fid) {
     return slot[fid];
 }
 
+// the cluster's levels with the case's sweeps and weights
+bool plan_coarse_levels(fvm_case* c, int S, bool exact, CoarsePlan& cp) {
+    std::vector<LevelDev> lv;
+    for (const DevLevel& L : c->levels) lv.push_back(L.dev);
+    if (!coarse_plan(lv, c->level_dir, c->inner, S, exact, cp)) return false;
+    const fvm_case_desc& d = c->desc;
+    cp.pre = d.coarse_sweeps > 0 ? d.coarse_sweeps : d.pre_sweeps;   // (levels below the finest)
+    cp.post = d.coarse_sweeps > 0 ? d.coarse_sweeps : d.post_sweeps;
+    cp.cheb = d.smoother == 1 ? 1 : 0;
+    if (cp.cheb)
+        for (int side = 0; side < 2; ++side) {
+            const int n = side ? cp.post : cp.pre;
+            for (int i = 0; i < n; ++i) cp.w[side][i] = sweep_weight(c, cp.lv[0].dev, n, i, side == 1);
+        }
+    return true;
+}
+
 fvm_status build_case(const Plan& pl, fvm_case* c) {
     const fvm_case_desc& d = pl.d;
     c->desc = d;
@@ -1255,35 +1277,24 @@ fvm_status build_case(const Plan& pl, fvm_case* c) {
         ST_TRY(dalloc(c, &D.e[1], v.N * si));
         ST_TRY(dalloc(c, &D.r, v.N * si));
     }
-    // the coarsest levels whose e, e', r fit in one CTA's shared memory (level 0 never does)
+    for (size_t l = 0; l < c->levels.size(); ++l) {
+        uint32_t m = 0;
+        for (int f = 0; f < 6; ++f)
+            if (std::find_if(pl.levels[l].dir[f].begin(), pl.levels[l].dir[f].end(), [](uint8_t x) { return x != 0; }) !=
+                pl.levels[l].dir[f].end())
+                m |= 1u << f;
+        c->level_dir.push_back(m);
+    }
+    // the largest cluster that the device runs
     {
-        // per cell: e, e', r in the compute type plus the 2-byte neighbour code.  FP64 runs
-        // at a small fraction of the FP32 rate on this part, so one SM only takes the
-        // last few hundred cells of an FP64 hierarchy
-        const size_t cs = (pl.inner == FVM_FP64 ? 8 : 4) * 3 + 2;
-        const size_t budget = pl.inner == FVM_FP64 ? 16 * 1024 : 200 * 1024;
-        size_t lc = c->levels.size() - 1;
-        size_t used = (size_t)c->levels[lc].dev.N * cs;
-        while (lc > 1 && used + (size_t)c->levels[lc - 1].dev.N * cs <= budget) {
-            --lc;
-            used += (size_t)c->levels[lc].dev.N * cs;
+        bool ok = false;
+        for (int S : {16, 8, 4, 2, 1}) {
+            if (!plan_coarse_levels(c, S, false, c->coarse)) continue;
+            if (prepare_coarse(pl.inner, c->coarse) != cudaSuccess) continue;
+            ok = true;
+            break;
         }
-        c->lc = lc;
-        memset(&c->coarse, 0, sizeof(c->coarse));
-        c->coarse.nl = (int)(c->levels.size() - lc);
-        c->coarse.pre = d.coarse_sweeps > 0 ? d.coarse_sweeps : d.pre_sweeps;   // (levels below the finest)
-        c->coarse.post = d.coarse_sweeps > 0 ? d.coarse_sweeps : d.post_sweeps;
-        for (int q = 0; q < c->coarse.nl; ++q) c->coarse.lv[q] = c->levels[lc + q].dev;
-        c->coarse.cheb = d.smoother == 1 ? 1 : 0;
-        if (c->coarse.cheb)
-            for (int side = 0; side < 2; ++side) {
-                const int n = side ? c->coarse.post : c->coarse.pre;
-                for (int i = 0; i < n; ++i) {
-                    c->coarse.w[side][i] = sweep_weight(c, c->coarse.lv[0], n, i, side == 1);
-                    c->coarse.wf[side][i] = (float)c->coarse.w[side][i];
-                }
-            }
-        CUDA_TRY(prepare_coarse_cta(pl.inner, coarse_cta_smem(c->coarse, pl.inner)));
+        if (!ok) return fail(FVM_ERR_CUDA, "the coarse-level kernel cannot run on this device");
     }
     // the paper's scheme applies the fine grid's stencil and diagonal on every level
     if (d.mg_variant == 1)
@@ -1629,6 +1640,10 @@ fvm_status batch_capture(fvm_batch* B, fvm_batch::Graph& G) {
         fvm_case* c = B->cases[i];
         save_ptrs(c, &G.before[12 * (size_t)i]);
         const int64_t launches0 = c->launches;
+        if (!plan_coarse_levels(c, coarse_cluster_for(n), true, c->coarse_many)) {
+            st = fail(FVM_ERR_INVALID, "batched case: no plan for its coarse levels");
+            break;
+        }
         Recorder R;
         g_rec = &R;
         for (int k : kStepStages)
