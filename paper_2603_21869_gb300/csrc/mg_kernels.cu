@@ -18,8 +18,8 @@
 // Every cell carries a 16-bit neighbour code (two bits per face: 0 = fluid
 // neighbour, 1 = zero-gradient ghost, 2 = zero-value ghost; bit 12 = solid),
 // so the stencil needs one small load instead of mask and face-table lookups.
-// Grid kernels use 3D blocks (no integer division).  All levels that fit in
-// one CTA's shared memory are cycled by a single CTA.  The level-0 residual
+// Grid kernels use 3D blocks (no integer division).  The coarse levels are
+// cycled by one cluster of blocks (coarse_kernels.cu).  The level-0 residual
 // kernel finishes the norm in its last block and decides on the device
 // whether another cycle runs, so the whole solve can live in a CUDA graph.
 #include "fvm_internal.cuh"
@@ -1765,8 +1765,9 @@ cudaError_t launch_resid0(int inner, int bprec, const LevelDev& L, const double*
     cudaError_t err = cudaSuccess;
     DISPATCH_I(inner, {
         if constexpr (sizeof(TI) < 8) {
-            // four cells per thread in float-float on large levels and in batches
-            if (bprec == FVM_FP32 && L.n[0] % 4 == 0 && (L.N >= (1 << 20) || g_rec)) {
+            // four cells per thread in float-float, whatever the size (430,080 cells: 47 us a launch in
+            // the one-cell form, which works in FP64)
+            if (bprec == FVM_FP32 && L.n[0] % 4 == 0) {
                 const int lrl = v4_lrl(L.n[0]);
                 int zc = 0;
                 const dim3 grid = v4_grid(L, lrl, zc);
@@ -1801,16 +1802,23 @@ static dim3 walk_grid(const LevelDev& L, int kz) {
 // block on grids too small for that).  The sweep aims for 16: it has no block reduction, and
 // shorter columns in more blocks balance better (the room's level-0 sweep: 42.3 us at four
 // planes a block, 37.3 at two, 40.0 at one); the kernels that end in a block reduction (the
-// residual, the inner products) aim for 8 (at two planes a block both measured about a third
-// slower, at eight or more planes a few per cent slower).
+// residual, the inner products) aim for 8 at 16 planes and more, for 1000 blocks (about two
+// waves) at 8, 4 and 2 planes, and take two planes rather than one from two blocks per SM on: a
+// block that reduces one plane's sums costs more than a second plane (ten steps of the
+// 256 x 64 x 64 FP32 channel 8.77 -> 8.19 ms from one plane to two; four of the 512 x 128 x 128
+// one 12.94 -> 12.84 ms from four planes to eight; 24 cycles of a 256 x 128 x 128 BF16 room 5.70
+// -> 5.60 ms from two planes to four; the 512 x 256 x 128 room at 16 planes instead of 8 54.3 ->
+// 55.1 ms; at two, both kernels a third slower).
 static int sweep_planes(int tiles, int nz, int fixed, int per_sm) {
     if (fixed > 0) return fixed < nz ? fixed : nz;
     // in a batch the cases' blocks add up: eight-plane columns (measured on 64 channels against
     // 4, 16 and 32: fewer re-read planes than 4, better balance than 16 or 32)
     if (g_rec) return nz < 8 ? nz : 8;
+    auto blocks = [&](int zc) { return tiles * ((nz + zc - 1) / zc); };
+    const bool reduces = per_sm <= 8;
     for (int zc : {32, 16, 8, 4, 2})
-        if (tiles * ((nz + zc - 1) / zc) >= per_sm * 152) return zc;
-    return 1;
+        if (blocks(zc) >= (reduces && zc <= 8 ? 1000 : per_sm * 152)) return zc;
+    return reduces && blocks(2) >= 2 * 152 ? 2 : 1;
 }
 
 // eight cells per thread on BF16 levels: in batches, and on single-case levels of 2^22 cells or
@@ -1931,7 +1939,10 @@ template <class TR, class TZ>
 static cudaError_t fcg_launch(const LevelDev& L, const TZ* z, const TR* r, TZ* dp, double* p, double* partials,
                               SolveState* st, cudaStream_t s) {
     if constexpr (sizeof(TR) < 8) {
-        if (L.n[0] % 4 == 0 && (L.N >= (1 << 20) || g_rec)) {
+        // (whatever the size: the one-cell pair, with its sums in FP64, took 58 us at 430,080 cells;
+        // this and the float-float residual together brought ten steps of that room from 18.9 to
+        // 13.4 ms)
+        if (L.n[0] % 4 == 0) {
             // (at most level0_blocks_max(n) blocks: partials has room)
             int zc = 0;
             constexpr int W = std::is_same<TR, TZ>::value ? vec_w<TR>() : 4;
