@@ -348,8 +348,8 @@ cudaError_t launch_unpack(int prec, const double* src, void* dst, int64_t N, cud
 // levels), bprec = storage type of b
 cudaError_t launch_solve_begin(SolveState* st, cudaStream_t s);
 cudaError_t launch_resid0(int inner, int bprec, const LevelDev& L, const double* p, const void* b, void* r, void* e,
-                          double* partials, SolveState* st, cudaGraphConditionalHandle cond,
-                          cudaGraphConditionalHandle cond2, int use_cond, cudaStream_t s);
+                          double* partials, SolveState* st, cudaGraphConditionalHandle cond, int use_cond,
+                          cudaStream_t s);
 cudaError_t launch_sweep_first(int inner, const LevelDev& L, const void* r, void* e, const SolveState* st,
                                cudaStream_t s);
 cudaError_t launch_sweep(int inner, const LevelDev& L, const void* e_in, const void* r, void* e_out,
@@ -545,19 +545,16 @@ struct BatchCtl {
     unsigned* counter;        // blocks finished in this launch (reset by the last one)
     SolveState* const* st;    // every case's solve state (device array)
     int n;
-    cudaGraphConditionalHandle cond, cond2;
-    int use_cond;             // 0: none, 1: cond, 2: cond and cond2
+    cudaGraphConditionalHandle cond;
+    int use_cond;             // 0: the host drives the loop
 };
 
 template <class K>
 __global__ void __launch_bounds__(K::kThreads, MinBlocks<K>::value) k_one_r0(const __grid_constant__ K k, cudaGraphConditionalHandle cond,
-                                                        cudaGraphConditionalHandle cond2, int use_cond) {
+                                                        int use_cond) {
     pdl_enter();
     const int go = k.run(BlockAt{blockIdx, gridDim});   // >= 0 only in the deciding thread
-    if (go >= 0 && use_cond) {
-        cudaGraphSetConditional(cond, go ? 1u : 0u);
-        if (use_cond > 1) cudaGraphSetConditional(cond2, go ? 1u : 0u);
-    }
+    if (go >= 0 && use_cond) cudaGraphSetConditional(cond, go ? 1u : 0u);
 }
 
 template <class K>
@@ -571,10 +568,7 @@ __global__ void __launch_bounds__(K::kThreads, MinBlocksMany<K>::value) k_many_r
     int any = 0;
     for (int i = 0; i < ctl.n; ++i) any |= ((volatile SolveState*)ctl.st[i])->active;
     *ctl.counter = 0u;
-    if (ctl.use_cond) {
-        cudaGraphSetConditional(ctl.cond, any ? 1u : 0u);
-        if (ctl.use_cond > 1) cudaGraphSetConditional(ctl.cond2, any ? 1u : 0u);
-    }
+    if (ctl.use_cond) cudaGraphSetConditional(ctl.cond, any ? 1u : 0u);
 }
 
 // Launch with the programmatic-serialization attribute (off when FVM_NO_PDL is set).
@@ -694,10 +688,10 @@ cudaError_t launch_k_one(const K& k, dim3 grid, dim3 block, size_t smem, cudaStr
 }
 
 template <class K>
-cudaError_t launch_r0(const K& k, dim3 grid, dim3 block, cudaGraphConditionalHandle cond,
-                      cudaGraphConditionalHandle cond2, int use_cond, cudaStream_t s) {
+cudaError_t launch_r0(const K& k, dim3 grid, dim3 block, cudaGraphConditionalHandle cond, int use_cond,
+                      cudaStream_t s) {
     if (record_launch(k, grid, block, 0, &many_launch_r0<K>)) return cudaSuccess;
-    return launch_pdl(k_one_r0<K>, grid, block, 0, s, k, cond, cond2, use_cond);
+    return launch_pdl(k_one_r0<K>, grid, block, 0, s, k, cond, use_cond);
 }
 
 // message returned by fvm_last_error() on this thread

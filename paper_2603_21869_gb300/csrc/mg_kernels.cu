@@ -1760,8 +1760,8 @@ static dim3 vw_grid(const LevelDev& L, int W, int lrl, int& zc, int per_sm = 8) 
 static dim3 v4_grid(const LevelDev& L, int lrl, int& zc) { return vw_grid(L, 4, lrl, zc); }
 
 cudaError_t launch_resid0(int inner, int bprec, const LevelDev& L, const double* p, const void* b, void* r, void* e,
-                          double* partials, SolveState* st, cudaGraphConditionalHandle cond,
-                          cudaGraphConditionalHandle cond2, int use_cond, cudaStream_t s) {
+                          double* partials, SolveState* st, cudaGraphConditionalHandle cond, int use_cond,
+                          cudaStream_t s) {
     cudaError_t err = cudaSuccess;
     DISPATCH_I(inner, {
         if constexpr (sizeof(TI) < 8) {
@@ -1773,15 +1773,15 @@ cudaError_t launch_resid0(int inner, int bprec, const LevelDev& L, const double*
                 const dim3 grid = v4_grid(L, lrl, zc);
                 // (at most level0_blocks_max(n) blocks: partials has room)
                 return launch_r0(Resid0V4K<TI>{L, p, (const float*)b, (TI*)r, (TI*)e, partials, st, zc, lrl}, grid,
-                                 dim3(TX, TY), cond, cond2, use_cond, s);
+                                 dim3(TX, TY), cond, use_cond, s);
             }
         }
         if (bprec == FVM_FP64)
             err = launch_r0(Resid0K<double, TI>{L, p, (const double*)b, (TI*)r, (TI*)e, partials, st}, grid3(L),
-                            kBlock3, cond, cond2, use_cond, s);
+                            kBlock3, cond, use_cond, s);
         else
             err = launch_r0(Resid0K<float, TI>{L, p, (const float*)b, (TI*)r, (TI*)e, partials, st}, grid3(L),
-                            kBlock3, cond, cond2, use_cond, s);
+                            kBlock3, cond, use_cond, s);
     });
     return err;
 }
