@@ -413,14 +413,22 @@ struct BatchMap {
     int total;           // start[n]: the cases' blocks together
 };
 
+// the last case whose first block is <= blk, found by a whole warp at once: its lanes look at 32
+// cases each with one load (a binary search is a chain of dependent loads before any work starts).
+// Blocks of less than a warp (one-thread launches) look case by case.
+template <bool Warp>
 __device__ __forceinline__ int batch_case(const BatchMap& m, int blk) {
-    int lo = 0, hi = m.n - 1;   // last case whose first block is <= blk
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(m.start + mid) <= blk) lo = mid;
-        else hi = mid - 1;
+    int at = 0;
+    if constexpr (Warp) {
+        const int lane = threadIdx.x & 31;   // (every block's x extent is a multiple of 32)
+        for (int q = 0; q < m.n; q += 32) {
+            const bool le = q + lane < m.n && __ldg(m.start + q + lane) <= blk;
+            at += __popc(__ballot_sync(0xffffffffu, le));
+        }
+    } else {
+        while (at < m.n && __ldg(m.start + at) <= blk) ++at;
     }
-    return lo;
+    return at - 1;   // (start[0] = 0)
 }
 
 // blocks per SM a functor asks the register allocator to keep resident (K::kMinBlocks, default 1)
@@ -449,20 +457,20 @@ __global__ void __launch_bounds__(K::kThreads, MinBlocks<K>::value) k_one(const 
     k.run(BlockAt{blockIdx, gridDim});
 }
 
-// Batched launches are persistent: block i takes the contiguous range
-// [i*per, (i+1)*per) of the cases' blocks, walks it with an incremental block
-// position, and copies a case's functor into shared memory when it enters
+// Batched launches: block i of g takes the i-th of g equal contiguous ranges
+// of the cases' blocks, walks it with an incremental block position, and copies a case's functor into shared memory when it enters
 // that case (skipping the case's blocks if it is no longer live).
 template <class K>
-__device__ __forceinline__ void batch_enter(const K* __restrict__ ks, const BatchMap& m, int c, unsigned char* buf,
-                                            int* s_live) {
+__device__ __forceinline__ void batch_fetch(const K* __restrict__ ks, int c, unsigned char* buf) {
     const int nt = blockDim.x * blockDim.y * blockDim.z;
     const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
-    __syncthreads();   // the previous functor is no longer read
     const uint32_t* src = (const uint32_t*)(ks + c);
     for (int q = tid; q < (int)(sizeof(K) / 4); q += nt) ((uint32_t*)buf)[q] = __ldg(src + q);
+}
+template <class K>
+__device__ __forceinline__ void batch_live(const unsigned char* buf, int* s_live) {
     __syncthreads();
-    if (tid == 0) *s_live = reinterpret_cast<const K*>(buf)->live() ? 1 : 0;
+    if (threadIdx.x + threadIdx.y + threadIdx.z == 0) *s_live = reinterpret_cast<const K*>(buf)->live() ? 1 : 0;
     __syncthreads();
 }
 
@@ -489,15 +497,20 @@ __device__ __forceinline__ void batch_run(const K* __restrict__ ks, const BatchM
     static_assert(sizeof(K) % 4 == 0, "functor size");
     __shared__ __align__(16) unsigned char buf[sizeof(K)];
     __shared__ int s_live;
-    const int per = (m.total + (int)gridDim.x - 1) / (int)gridDim.x;
-    const int lo = (int)blockIdx.x * per, hi = min(m.total, lo + per);
-    if (lo >= hi) return;
-    int c = batch_case(m, lo);
+    const int lo = (int)((int64_t)blockIdx.x * m.total / (int)gridDim.x);
+    const int hi = (int)((int64_t)(blockIdx.x + 1) * m.total / (int)gridDim.x);
+    if (lo >= hi) {
+        pdl_enter();
+        return;
+    }
+    int c = batch_case<(K::kThreads >= 32)>(m, lo);
+    batch_fetch(ks, c, buf);
     uint3 g = m.grid[c];
     unsigned l = (unsigned)(lo - __ldg(m.start + c));
     uint3 b = make_uint3(l % g.x, (l / g.x) % g.y, l / (g.x * g.y));
     int cend = __ldg(m.start + c + 1);
-    batch_enter(ks, m, c, buf, &s_live);
+    pdl_enter();
+    batch_live<K>(buf, &s_live);
     for (int v = lo; v < hi; ++v) {
         if (v == cend) {   // the next case with blocks begins at its own first block
             do {           // (the host rejects empty cases; skipping them keeps the walk in bounds anyway)
@@ -506,7 +519,9 @@ __device__ __forceinline__ void batch_run(const K* __restrict__ ks, const BatchM
             } while (v == cend);
             g = m.grid[c];
             b = make_uint3(0, 0, 0);
-            batch_enter(ks, m, c, buf, &s_live);
+            __syncthreads();   // the previous functor is no longer read
+            batch_fetch(ks, c, buf);
+            batch_live<K>(buf, &s_live);
         }
         if (s_live) {
             batch_block_body(*reinterpret_cast<const K*>(buf), BlockAt{b, g});
@@ -534,7 +549,6 @@ struct MinBlocksMany<K, std::void_t<decltype(K::kMinBlocksMany)>> {
 
 template <class K>
 __global__ void __launch_bounds__(K::kThreads, MinBlocksMany<K>::value) k_many(const K* __restrict__ ks, BatchMap m) {
-    pdl_enter();
     batch_run(ks, m);
 }
 
@@ -559,7 +573,6 @@ __global__ void __launch_bounds__(K::kThreads, MinBlocks<K>::value) k_one_r0(con
 
 template <class K>
 __global__ void __launch_bounds__(K::kThreads, MinBlocksMany<K>::value) k_many_r0(const K* __restrict__ ks, BatchMap m, BatchCtl ctl) {
-    pdl_enter();
     batch_run(ks, m);
     if (threadIdx.x + threadIdx.y + threadIdx.z != 0) return;
     __threadfence();   // the decisions this block made, before the count
@@ -609,6 +622,7 @@ struct Recorder {
     std::vector<RecLaunch> out;
     std::string site;                  // set by the caller before each launch site
     double bytes = 0.0;                // algorithmic bytes of the site (given to its first launch)
+    int cases = 1;                     // cases of the batch being recorded
 };
 
 extern thread_local Recorder* g_rec;
@@ -622,7 +636,7 @@ cudaError_t raise_smem_limit(const void* fn, size_t bytes);
 // a launch brought the process down).
 bool smem_limit_covers(const void* fn, size_t bytes);
 
-// Blocks of a persistent batched launch: the SMs times the blocks of this
+// Resident blocks of a batched launch: the SMs times the blocks of this
 // kernel that fit on one SM (queried once per kernel and shared-memory size,
 // outside any capture, when `query` is set).
 int persistent_blocks(const void* fn, int threads, size_t smem, bool query);
@@ -642,7 +656,12 @@ cudaError_t many_launch(const void* tab, const BatchMap& m, unsigned nblk, dim3 
     if (!smem_limit_covers(fn, smem)) return cudaErrorInvalidConfiguration;
     const int pb = persistent_blocks(fn, threads, smem, false);
     if (pb <= 0) return cudaErrorInvalidConfiguration;
-    return launch_pdl(k_many<K>, dim3(nblk < (unsigned)pb ? nblk : (unsigned)pb), block, smem, s, (const K*)tab, m);
+    // six rounds of resident blocks at most: in one round a block that draws the long end of its
+    // range holds up the launch (8 served BF16 cases 50.2 -> 44 ms, 64 channels 21.4 -> 19.4 ms a
+    // step at eight planes a column; without a limit the small cases' blocks each fetch a functor
+    // and 8 channels lose 5 %)
+    const unsigned most = 6u * (unsigned)pb;
+    return launch_pdl(k_many<K>, dim3(nblk < most ? nblk : most), block, smem, s, (const K*)tab, m);
 }
 
 template <class K>

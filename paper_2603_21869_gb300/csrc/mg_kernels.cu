@@ -1747,14 +1747,14 @@ cudaError_t launch_solve_begin(SolveState* st, cudaStream_t s) {
     return launch_k(SolveBeginK{st}, dim3(1), dim3(1), 0, s);
 }
 
-static int sweep_planes(int tiles, int nz, int fixed, int per_sm);
+static int sweep_planes(int tiles, int nz, int fixed, int per_sm, int W);
 
 // vector kernels: the block's x-y extent for W cells per thread and the row segments of lrl;
 // per_sm: the blocks per SM the plane rule aims for
 static dim3 vw_grid(const LevelDev& L, int W, int lrl, int& zc, int per_sm = 8) {
     const int wx = W << lrl, wy = TY << (5 - lrl);
     const int tiles = ((L.n[0] + wx - 1) / wx) * ((L.n[1] + wy - 1) / wy);
-    zc = sweep_planes(tiles, L.n[2], L.zc_fixed, per_sm);
+    zc = sweep_planes(tiles, L.n[2], L.zc_fixed, per_sm, W);
     return dim3((unsigned)((L.n[0] + wx - 1) / wx), (unsigned)((L.n[1] + wy - 1) / wy), (unsigned)((L.n[2] + zc - 1) / zc));
 }
 static dim3 v4_grid(const LevelDev& L, int lrl, int& zc) { return vw_grid(L, 4, lrl, zc); }
@@ -1809,12 +1809,21 @@ static dim3 walk_grid(const LevelDev& L, int kz) {
 // one 12.94 -> 12.84 ms from four planes to eight; 24 cycles of a 256 x 128 x 128 BF16 room 5.70
 // -> 5.60 ms from two planes to four; the 512 x 256 x 128 room at 16 planes instead of 8 54.3 ->
 // 55.1 ms; at two, both kernels a third slower).
-static int sweep_planes(int tiles, int nz, int fixed, int per_sm) {
+static int sweep_planes(int tiles, int nz, int fixed, int per_sm, int W) {
     if (fixed > 0) return fixed < nz ? fixed : nz;
-    // in a batch the cases' blocks add up: eight-plane columns (measured on 64 channels against
-    // 4, 16 and 32: fewer re-read planes than 4, better balance than 16 or 32)
-    if (g_rec) return nz < 8 ? nz : 8;
     auto blocks = [&](int zc) { return tiles * ((nz + zc - 1) / zc); };
+    if (g_rec) {
+        // in a batch the cases' blocks add up (taken as all of this case's size): the longest columns
+        // of at most eight planes that leave the launch this many blocks, fewer for the kernels that
+        // end in a block reduction and more for the eight-cell sweep (two planes of a small level's
+        // block take longer than the level: with eight-plane columns throughout, 8 FP32 channels
+        // took 14.8 ms for four steps against 13.6 ms, 8 served BF16 cases 43.9 against 34.0 ms for
+        // two; 64 channels 19.4 ms a step either way)
+        const int want = per_sm <= 8 ? 300 : (W == 8 ? 1500 : 608);
+        for (int zc : {8, 4, 2})
+            if ((int64_t)blocks(zc) * g_rec->cases >= want) return nz < zc ? nz : zc;
+        return 1;
+    }
     const bool reduces = per_sm <= 8;
     for (int zc : {32, 16, 8, 4, 2})
         if (blocks(zc) >= (reduces && zc <= 8 ? 1000 : per_sm * 152)) return zc;

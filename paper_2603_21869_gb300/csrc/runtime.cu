@@ -1634,6 +1634,7 @@ fvm_status batch_capture(fvm_batch* B, fvm_batch::Graph& G) {
             break;
         }
         Recorder R;
+        R.cases = n;
         g_rec = &R;
         for (int k : kStepStages)
             if (st == FVM_OK) st = stage(c, k, nullptr, nullptr);
