@@ -1389,6 +1389,7 @@ __device__ void Lambda2K<S, C>::run(const BlockAt& at) const {
     }
     // only u, v, w of the loaded states are used; the other loads are dead code
     const St<C> P = load_state<S, C>(in, c);
+    const bool reg = regular_cell(cd, c);
     C g[3][3];   // g[a][b] = d u_a / d x_b
     for (int b = 0; b < 3; ++b) {
         if (!cd.active[b]) {
@@ -1396,8 +1397,13 @@ __device__ void Lambda2K<S, C>::run(const BlockAt& at) const {
             continue;
         }
         St<C> L, R;
-        neighbour<S, C>(cd, in, i, j, k, b, -1, P, L);
-        neighbour<S, C>(cd, in, i, j, k, b, +1, P, R);
+        if (reg) {
+            L = regular_neighbour<S, C>(cd, in, i, j, k, b, -1);
+            R = regular_neighbour<S, C>(cd, in, i, j, k, b, +1);
+        } else {
+            neighbour<S, C>(cd, in, i, j, k, b, -1, P, L);
+            neighbour<S, C>(cd, in, i, j, k, b, +1, P, R);
+        }
         const C ih = prm<C>(cd.inv_h[b], cd.f.inv_h[b]);
         g[0][b] = (C)0.5 * ((R.u - P.u) * ih + (P.u - L.u) * ih);
         g[1][b] = (C)0.5 * ((R.v - P.v) * ih + (P.v - L.v) * ih);
