@@ -366,8 +366,8 @@ __device__ __forceinline__ bool walk_setup(const LevelDev& L, const BlockAt& at,
     return true;
 }
 
-// Scalar sweep (FP64 levels, and levels whose x extent is not a multiple of
-// 4): each thread walks KZ cells along z, keeping the z neighbours in
+// Scalar sweep (FP32 and BF16 levels under 2^20 cells of a case alone or with an x extent that is
+// not a multiple of 4, FP64 levels with a collapsed x axis): each thread walks KZ cells along z, keeping the z neighbours in
 // registers; all loads of its cells are issued before any arithmetic.
 // MODE 0: eout = sweep(ein); MODE 1: p += sweep(ein) (last level-0 sweep); MODE 2: the
 // result in FP32 (the last level-0 sweep under the flexible-CG acceleration of BF16 levels).
@@ -432,8 +432,8 @@ __device__ void SweepK<TI, MODE, KZ>::run(const BlockAt& at) const {
     }
 }
 
-// W consecutive x cells per thread (the vector kernels): W = 4 with 128-bit
-// loads for FP32 levels, W = 8 with 128-bit loads for BF16 levels (W = 4,
+// W consecutive x cells per thread (the vector kernels): W = 2 with 128-bit
+// loads for FP64 levels, W = 4 for FP32 levels, W = 8 with 128-bit loads for BF16 levels (W = 4,
 // 64-bit loads, where nx is not a multiple of 8).  A warp covers W * 32
 // cells of a row (or 2, 4, 8 rows of W * 16, W * 8, W * 4 cells: the widest
 // segment that divides nx) and marches zc planes in z: rows j +- 1 and the
@@ -506,6 +506,19 @@ template <> struct VecW<__nv_bfloat16, 8> {
             make_uint4(bf2_pack(v[0], v[1]), bf2_pack(v[2], v[3]), bf2_pack(v[4], v[5]), bf2_pack(v[6], v[7]));
     }
 };
+template <> struct VecW<double, 2> {
+    static __device__ __forceinline__ void load_rw(const double* p, int c, double (&o)[2]) {
+        const double2 v = *reinterpret_cast<const double2*>(p + c);
+        o[0] = v.x; o[1] = v.y;
+    }
+    static __device__ __forceinline__ void load(const double* p, int c, double (&o)[2]) {
+        const double2 v = __ldg(reinterpret_cast<const double2*>(p + c));
+        o[0] = v.x; o[1] = v.y;
+    }
+    static __device__ __forceinline__ void store(double* p, int c, const double (&v)[2]) {
+        *reinterpret_cast<double2*>(p + c) = make_double2(v[0], v[1]);
+    }
+};
 // the four-cell loads of the other kernels
 template <class TI> using Vec4 = VecW<TI, 4>;
 
@@ -521,13 +534,16 @@ template <> __device__ __forceinline__ void codes_w<8>(const uint16_t* f, int c,
     o[4] = v.z & 0xffffu; o[5] = v.z >> 16; o[6] = v.w & 0xffffu; o[7] = v.w >> 16;
 }
 
+template <> __device__ __forceinline__ void codes_w<1>(const uint16_t* f, int c, uint32_t (&o)[1]) {
+    o[0] = __ldg(f + c);
+}
 template <> __device__ __forceinline__ void codes_w<2>(const uint16_t* f, int c, uint32_t (&o)[2]) {
     const uint32_t v = __ldg(reinterpret_cast<const unsigned int*>(f + c));
     o[0] = v & 0xffffu; o[1] = v >> 16;
 }
 
 // cells per thread of the vector kernels on a level of this storage type
-template <class TI> __device__ __host__ constexpr int vec_w() { return sizeof(TI) == 2 ? 8 : 4; }
+template <class TI> __device__ __host__ constexpr int vec_w() { return sizeof(TI) == 2 ? 8 : (sizeof(TI) == 4 ? 4 : 2); }
 
 // The register image of W cells as loaded (16 bytes for W = 4 FP32 and W = 8
 // BF16), converted to FP32 one value at a time where used: keeps the vector
@@ -576,6 +592,47 @@ template <> struct RawW<__nv_bfloat16, 8> {
     }
 };
 
+template <> struct RawW<double, 2> {
+    using T = double2;
+    static __device__ __forceinline__ T load(const double* p, int c) { return __ldg(reinterpret_cast<const double2*>(p + c)); }
+    static __device__ __forceinline__ double get(const T& v, int t) { return t == 0 ? v.x : v.y; }
+};
+template <> struct RawW<double, 1> {
+    using T = double;
+    static __device__ __forceinline__ T load(const double* p, int c) { return __ldg(p + c); }
+    static __device__ __forceinline__ double get(const T& v, int) { return v; }
+};
+
+// FP64 levels (two cells per thread) are bound by the FP64 pipe, two lanes a clock and SM: ghosts
+// are chosen by integer operations (a negation that no instruction takes as a modifier, like a
+// second pass over a warp with one irregular cell, costs FP64 instructions), and the stencil takes
+// 8 operations a cell, r - A e summed from r on: fma(-diag, e_P, r + sum_a ih_a (lo + hi)).
+// Measured against one cell per thread at 256 x 64 x 64 cells: sweep 38.5 -> 23.1 us, residual 70 ->
+// 38.8, residual and restriction 38.9 -> 26.9, prolongation 61.5 -> 43.0; the sweep's 8 operations
+// are 13.3 us at the pipe's rate.
+__device__ __forceinline__ double flipped(double x, bool neg) {
+    return __hiloint2double(__double2hiint(x) ^ (int)((unsigned)neg << 31), __double2loint(x));
+}
+__device__ __forceinline__ double ghost64(uint32_t code, double nb, double eP) {   // (code: the face's two bits)
+    return code == 0u ? nb : flipped(eP, code == 2u);
+}
+// r - A e at one cell, every neighbour as loaded at clamped indices
+__device__ __forceinline__ double resid64(uint32_t f, double r, double eP, double xm, double xp, double ym, double yp,
+                                          double zm, double zp, double ihx, double ihy, double ihz, double dg) {
+    if (f & 0x2000u) {
+        xm = ghost64(f & 3u, xm, eP);
+        xp = ghost64((f >> 2) & 3u, xp, eP);
+        ym = ghost64((f >> 4) & 3u, ym, eP);
+        yp = ghost64((f >> 6) & 3u, yp, eP);
+        zm = ghost64((f >> 8) & 3u, zm, eP);
+        zp = ghost64((f >> 10) & 3u, zp, eP);
+    }
+    double s = fma(xm + xp, ihx, r);
+    s = fma(ym + yp, ihy, s);
+    s = fma(zm + zp, ihz, s);
+    return fma(-dg, eP, s);
+}
+
 // Ask L2 for the line holding p (no register is tied up while it lands): the z-march kernels
 // name their rows of the plane three ahead, so that those loads later hit L2 instead of
 // waiting out a DRAM round trip.
@@ -607,7 +664,7 @@ struct SweepVK {
 
 template <class TI, int MODE, int W>
 __device__ void SweepVK<TI, MODE, W>::run(const BlockAt& at) const {
-    using C = float;
+    using C = typename Acc<TI>::type;
     const int nx = L.n[0], ny = L.n[1], nz = L.n[2];
     const int LR = 1 << lrl, lane = threadIdx.x & (LR - 1), sub = threadIdx.x >> lrl;
     const int i4 = at.b.x * (W * LR) + lane * W, j = ((at.b.y * TY + threadIdx.y) << (5 - lrl)) + sub;
@@ -657,7 +714,16 @@ __device__ void SweepVK<TI, MODE, W>::run(const BlockAt& at) const {
         uint32_t any = 0u;   // solid (bit 12) or irregular (bit 13) anywhere among the W cells
 #pragma unroll
         for (int t = 0; t < W; ++t) any |= fs[t];
-        if (!(any & 0x3000u)) {
+        if constexpr (sizeof(C) == 8) {
+#pragma unroll
+            for (int t = 0; t < W; ++t) {
+                const C eP = R::get(ec, t);
+                const C d = resid64(fs[t], R::get(rr, t), eP, t == 0 ? left : R::get(ec, t - 1),
+                                    t == W - 1 ? right : R::get(ec, t + 1), R::get(ym, t), R::get(yp, t), R::get(em, t),
+                                    R::get(ep, t), ihx, ihy, ihz, dg);
+                v[t] = is_solid(fs[t]) ? (C)0 : fma(wiD, d, eP);
+            }
+        } else if (!(any & 0x3000u)) {
             // every cell fluid, each ghost the clamped in-grid load: the plain stencil
 #pragma unroll
             for (int t = 0; t < W; ++t) {
@@ -687,10 +753,16 @@ __device__ void SweepVK<TI, MODE, W>::run(const BlockAt& at) const {
             }
         }
         if (in) {
-            if (MODE == 0) {
+            if constexpr (MODE == 0) {
                 VecW<TI, W>::store(eout, base + own, v);
-            } else if (MODE == 2) {
+            } else if constexpr (MODE == 2) {
                 VecW<float, W>::store(z32, base + own, v);
+            } else if constexpr (sizeof(C) == 8) {
+                double o[W];
+                VecW<double, W>::load_rw(p, base + own, o);
+#pragma unroll
+                for (int t = 0; t < W; ++t) o[t] = o[t] + v[t];   // (0 in solid cells)
+                VecW<double, W>::store(p, base + own, o);
             } else {   // p (double-float pairs) += the correction, two cells per 16 bytes
                 float4* pp = reinterpret_cast<float4*>(p + base + own);
 #pragma unroll
@@ -898,6 +970,40 @@ template <> __device__ __forceinline__ float round_inner<__nv_bfloat16>(float v)
     return __bfloat162float(__float2bfloat16_rn(v));
 }
 
+// block sums in FP64, then the last block's fixed-order reduction and the stopping rule (the
+// decision in the deciding thread, -1 elsewhere)
+template <int NT>
+__device__ __forceinline__ int resid0_sums(double s0, double s1, double* partials, SolveState* st, const BlockAt& at) {
+    __shared__ double red[2][NT / 32];
+    __shared__ bool last;
+    const int tid = threadIdx.x + TX * threadIdx.y;
+    for (int off = 16; off > 0; off >>= 1) {
+        s0 += __shfl_xor_sync(0xffffffffu, s0, off);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, off);
+    }
+    if ((tid & 31) == 0) {
+        red[0][tid >> 5] = s0;
+        red[1][tid >> 5] = s1;
+    }
+    __syncthreads();
+    const int nblk = at.g.x * at.g.y * at.g.z;
+    if (tid == 0) {
+        const int bid = at.b.x + at.g.x * (at.b.y + at.g.y * at.b.z);
+        double a0 = 0.0, a1 = 0.0;
+        for (int w = 0; w < NT / 32; ++w) {
+            a0 += red[0][w];
+            a1 += red[1][w];
+        }
+        reinterpret_cast<double2*>(partials)[bid] = make_double2(a0, a1);
+        __threadfence();
+        last = atomicAdd(&st->counter, 1u) == (unsigned)nblk - 1u;
+    }
+    __syncthreads();
+    if (!last) return -1;
+    __threadfence();
+    return resid0_finish<NT>(partials, nblk, st, red);
+}
+
 // r = b - A p (float-float), r^2 and b^2, the first pre-sweep e = w_J r / D;
 // four x cells per thread and a z march (the sweep's layout).  FP32 b, nx % 4 = 0.
 template <class TI>
@@ -1022,36 +1128,63 @@ __device__ int Resid0V4K<TI>::run(const BlockAt& at) const {
             ep[t] = en[t];
         }
     }
-    // block sums in FP64, then the last block's fixed-order reduction and the stopping rule
-    __shared__ double red[2][kThreads / 32];
-    __shared__ bool last;
-    const int tid = threadIdx.x + TX * threadIdx.y;
-    double s0 = (double)r2, s1 = (double)b2;
-    for (int off = 16; off > 0; off >>= 1) {
-        s0 += __shfl_xor_sync(0xffffffffu, s0, off);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, off);
-    }
-    if ((tid & 31) == 0) {
-        red[0][tid >> 5] = s0;
-        red[1][tid >> 5] = s1;
-    }
-    __syncthreads();
-    const int nblk = at.g.x * at.g.y * at.g.z;
-    if (tid == 0) {
-        const int bid = at.b.x + at.g.x * (at.b.y + at.g.y * at.b.z);
-        double a0 = 0.0, a1 = 0.0;
-        for (int w = 0; w < kThreads / 32; ++w) {
-            a0 += red[0][w];
-            a1 += red[1][w];
+    return resid0_sums<kThreads>((double)r2, (double)b2, partials, st, at);
+}
+
+// r = b - A p, r^2 and b^2 and the first pre-sweep of an FP64 level: two x cells per thread and a z
+// march (the sweep's layout); a thread's squares are summed in registers, one warp reduction a block
+// (the one-cell form's per-cell reduction was 10 of its 24 FP64 operations a cell).
+struct Resid0D2K {
+    static constexpr int kThreads = TX * TY;
+    static constexpr int kMinBlocks = 4;
+    LevelDev L;
+    const double* p;
+    const double* b;
+    double* r;
+    double* e;
+    double* partials;
+    SolveState* st;
+    int zc;    // planes per block
+    int lrl;   // log2 of the lanes per row segment (as in SweepVK)
+    __device__ bool live() const { return st->active != 0; }
+    __device__ int run(const BlockAt& at) const;
+};
+
+__device__ int Resid0D2K::run(const BlockAt& at) const {
+    using R = RawW<double, 2>;
+    const int nx = L.n[0], ny = L.n[1], nz = L.n[2];
+    const int LR = 1 << lrl, lane = threadIdx.x & (LR - 1), sub = threadIdx.x >> lrl;
+    const int i2 = at.b.x * (2 * LR) + lane * 2, j = ((at.b.y * TY + threadIdx.y) << (5 - lrl)) + sub;
+    const int k0 = at.b.z * zc, k1 = min(nz, k0 + zc);
+    const bool in = i2 < nx && j < ny;
+    const int sy = nx, sz = nx * ny;
+    const int ic = min(i2, nx - 2), jc = min(j, ny - 1);
+    const int own = ic + sy * jc, om = ic + sy * max(jc - 1, 0), op = ic + sy * min(jc + 1, ny - 1);
+    const int xl = max(ic - 1, 0) + sy * jc, xr = min(ic + 2, nx - 1) + sy * jc;
+    const double ihx = L.ih2a[0], ihy = L.ih2a[1], ihz = L.ih2a[2], dg = L.diag, wiD = L.wJ * L.inv_D;
+    double2 em = R::load(p, max(k0 - 1, 0) * sz + own), ec = R::load(p, k0 * sz + own);
+    double r2 = 0.0, b2 = 0.0;
+    for (int k = k0; k < k1; ++k) {
+        const int base = k * sz;
+        const double2 ep = R::load(p, min(k + 1, nz - 1) * sz + own);
+        const double2 ym = R::load(p, base + om), yp = R::load(p, base + op), bv = R::load(b, base + own);
+        const double left = __ldg(p + base + xl), right = __ldg(p + base + xr);
+        uint32_t fs[2];
+        codes_w<2>(L.nbf, base + own, fs);
+        const double a = resid64(fs[0], bv.x, ec.x, left, ec.y, ym.x, yp.x, em.x, ep.x, ihx, ihy, ihz, dg);
+        const double c = resid64(fs[1], bv.y, ec.y, ec.x, right, ym.y, yp.y, em.y, ep.y, ihx, ihy, ihz, dg);
+        const double ra = is_solid(fs[0]) ? 0.0 : a, rc = is_solid(fs[1]) ? 0.0 : c;
+        if (in) {
+            *reinterpret_cast<double2*>(r + base + own) = make_double2(ra, rc);
+            *reinterpret_cast<double2*>(e + base + own) = make_double2(wiD * ra, wiD * rc);
+            r2 = fma(ra, ra, fma(rc, rc, r2));
+            const double ba = is_solid(fs[0]) ? 0.0 : bv.x, bc = is_solid(fs[1]) ? 0.0 : bv.y;
+            b2 = fma(ba, ba, fma(bc, bc, b2));
         }
-        reinterpret_cast<double2*>(partials)[bid] = make_double2(a0, a1);
-        __threadfence();
-        last = atomicAdd(&st->counter, 1u) == (unsigned)nblk - 1u;
+        em = ec;
+        ec = ep;
     }
-    __syncthreads();
-    if (!last) return -1;
-    __threadfence();
-    return resid0_finish<kThreads>(partials, nblk, st, red);
+    return resid0_sums<kThreads>(r2, b2, partials, st, at);
 }
 
 // The flexible-CG inner products with W x cells per thread and a z march
@@ -1077,7 +1210,7 @@ struct FcgDotVK {
 
 template <class TR, class TZ, int W>
 __device__ void FcgDotVK<TR, TZ, W>::run(const BlockAt& at) const {
-    using C = float;
+    using C = typename Acc<TZ>::type;
     using R = RawW<TZ, W>;
     using RR = RawW<TR, W>;
     const int nx = L.n[0], ny = L.n[1], nz = L.n[2];
@@ -1098,7 +1231,7 @@ __device__ void FcgDotVK<TR, TZ, W>::run(const BlockAt& at) const {
     typename R::T em = R::load(zz, max(k0 - 1, 0) * sz + own);
     typename R::T ec = R::load(zz, k0 * sz + own);
     typename R::T ep = R::load(zz, min(k0 + 1, nz - 1) * sz + own);
-    C a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+    C a0 = (C)0, a1 = (C)0, a2 = (C)0, a3 = (C)0;
     for (int k = k0; k < k1; ++k) {
         const int base = k * sz;
         const typename R::T ym = R::load(zz, base + om);
@@ -1143,7 +1276,9 @@ __device__ void FcgDotVK<TR, TZ, W>::run(const BlockAt& at) const {
                 const C xm = t == 0 ? left : R::get(ec, t - 1), xp = t == W - 1 ? right : R::get(ec, t + 1);
                 const C ya = R::get(ym, t), yb = R::get(yp, t), za = R::get(em, t), zb = R::get(ep, t);
                 C A;
-                if (plain || !((fs[t] >> 13) & 1u)) {
+                if constexpr (sizeof(C) == 8) {
+                    A = -resid64(fs[t], 0.0, eP, xm, xp, ya, yb, za, zb, ihx, ihy, ihz, dg);
+                } else if (plain || !((fs[t] >> 13) & 1u)) {
                     C q = (xm + xp) * ihx;
                     q = fma(ya + yb, ihy, q);
                     q = fma(za + zb, ihz, q);
@@ -1162,7 +1297,7 @@ __device__ void FcgDotVK<TR, TZ, W>::run(const BlockAt& at) const {
         ec = ep;
         ep = en;
     }
-    float s[4] = {a0, a1, a2, a3};   // FP32 within a warp, FP64 from the warp sums on
+    C s[4] = {a0, a1, a2, a3};   // (FP32 corrections: FP32 within a warp, FP64 from the warp sums on)
     fcg_reduce<kThreads>(s, partials, st, have, at);
 }
 
@@ -1181,18 +1316,28 @@ struct FcgUpdVK {
     __device__ void run(const BlockAt& at) const {
         const int c = W * (at.b.x * kThreads + threadIdx.x);
         if (c >= L.N) return;
-        const float alpha = (float)st->g_alpha, beta = (float)st->g_beta;
-        float zv[W], dv[W];
+        using C = typename Acc<TZ>::type;
+        const C alpha = (C)st->g_alpha, beta = (C)st->g_beta;
+        C zv[W], dv[W];
 #pragma unroll
-        for (int t = 0; t < W; ++t) dv[t] = 0.f;
+        for (int t = 0; t < W; ++t) dv[t] = (C)0;
         VecW<TZ, W>::load(z, c, zv);
-        if (beta != 0.f) VecW<TZ, W>::load_rw(dp, c, dv);
+        if (beta != (C)0) VecW<TZ, W>::load_rw(dp, c, dv);
         uint32_t fs[W];
         codes_w<W>(L.nbf, c, fs);
-        float d[W];
+        C d[W];
 #pragma unroll
         for (int t = 0; t < W; ++t) d[t] = fma(-beta, dv[t], zv[t]);
         VecW<TZ, W>::store(dp, c, d);
+        if constexpr (sizeof(C) == 8) {
+            double u[W];
+            VecW<double, W>::load_rw(p, c, u);
+#pragma unroll
+            for (int t = 0; t < W; ++t)
+                if (!is_solid(fs[t])) u[t] = fma(alpha, d[t], u[t]);
+            VecW<double, W>::store(p, c, u);
+            return;
+        }
         float4* pp = reinterpret_cast<float4*>(p + c);   // p as double-float pairs, two cells per 16 bytes
 #pragma unroll
         for (int h = 0; h < W / 2; ++h) {
@@ -1236,7 +1381,8 @@ struct ProlongVK {
 };
 
 // a coarse value across a ghost row or plane: negated for each zero-value face among them
-__device__ __forceinline__ float ghost_signed(uint32_t code, bool gy, int sy, bool gz, int sz, float v) {
+template <class C>
+__device__ __forceinline__ C ghost_signed(uint32_t code, bool gy, int sy, bool gz, int sz, C v) {
     bool neg = gy && ((code >> (2 * (2 + sy))) & 3u) == 2u;
     neg ^= gz && ((code >> (2 * (4 + sz))) & 3u) == 2u;
     return neg ? -v : v;
@@ -1244,7 +1390,7 @@ __device__ __forceinline__ float ghost_signed(uint32_t code, bool gy, int sy, bo
 
 template <class TI, int W>
 __device__ void ProlongVK<TI, W>::run(const BlockAt& at) const {
-    using C = float;
+    using C = typename Acc<TI>::type;
     constexpr int H = W / 2;   // coarse cells under a thread's W fine cells
     using RC = RawW<TI, H>;
     const int nx = Lf.n[0], ny = Lf.n[1], nz = Lf.n[2];
@@ -1280,6 +1426,7 @@ __device__ void ProlongVK<TI, W>::run(const BlockAt& at) const {
         for (int h = 0; h < H; ++h) cvc[h] = (C)0;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
+            if ((q & 2) && !zact) continue;   // (a collapsed z axis: no second plane)
             const int jj = (q & 1) ? Qj : Pj, kk = (q & 2) ? Qk : Pk;
             const bool gy = (q & 1) && outJ, gz = (q & 2) && outK;
             const C w = ((q & 1) ? (C)0.25 : (C)0.75) * ((q & 2) ? wz1 : wz0);
@@ -1357,7 +1504,7 @@ struct RRVK {
 
 template <class TI, int W>
 __device__ void RRVK<TI, W>::run(const BlockAt& at) const {
-    using C = float;
+    using C = typename Acc<TI>::type;
     using R = RawW<TI, W>;
     constexpr int H = W / 2;
     const int nx = Lf.n[0], ny = Lf.n[1], nz = Lf.n[2];
@@ -1406,6 +1553,10 @@ __device__ void RRVK<TI, W>::run(const BlockAt& at) const {
                 const C eP = R::get(ec, t);
                 const C xm = t == 0 ? left : R::get(ec, t - 1), xp = t == W - 1 ? right : R::get(ec, t + 1);
                 const C ya = R::get(yl, t), yb = R::get(yh, t), za = R::get(zl, t), zb = R::get(zh, t);
+                if constexpr (sizeof(C) == 8) {
+                    s[t >> 1] += resid64(fs[t], R::get(rr, t), eP, xm, xp, ya, yb, za, zb, ihx, ihy, ihz, dg);
+                    continue;
+                }
                 C A;
                 if (!((fs[t] >> 13) & 1u)) {
                     C sa = (xm + xp) * ihx;
@@ -1728,7 +1879,7 @@ static int v4_lrl(int nx) { return vw_lrl(nx, 4); }
 int level0_blocks_max(int nx, int ny, int nz) {
     // a vector pass (four or eight cells per thread) with this nx's row segments, one plane a block
     int most = resid0_blocks(nx, ny, nz);
-    for (int W : {4, 8}) {
+    for (int W : {2, 4, 8}) {
         const int lrl = vw_lrl(nx, W), wx = W << lrl, wy = TY << (5 - lrl);
         const int n = ((nx + wx - 1) / wx) * ((ny + wy - 1) / wy) * nz;
         most = n > most ? n : most;
@@ -1773,6 +1924,15 @@ cudaError_t launch_resid0(int inner, int bprec, const LevelDev& L, const double*
                 const dim3 grid = v4_grid(L, lrl, zc);
                 // (at most level0_blocks_max(n) blocks: partials has room)
                 return launch_r0(Resid0V4K<TI>{L, p, (const float*)b, (TI*)r, (TI*)e, partials, st, zc, lrl}, grid,
+                                 dim3(TX, TY), cond, use_cond, s);
+            }
+        }
+        if constexpr (sizeof(TI) == 8) {
+            if (bprec == FVM_FP64 && L.n[0] % 2 == 0) {
+                const int lrl = vw_lrl(L.n[0], 2);
+                int zc = 0;
+                const dim3 grid = vw_grid(L, 2, lrl, zc);
+                return launch_r0(Resid0D2K{L, p, (const double*)b, (double*)r, (double*)e, partials, st, zc, lrl}, grid,
                                  dim3(TX, TY), cond, use_cond, s);
             }
         }
@@ -1854,6 +2014,14 @@ static cudaError_t sweep_walk(const LevelDev& L, const TI* ein, const TI* r, TI*
             return launch_k(SweepVK<TI, MODE, 4>{L, ein, r, eout, p, st, zc, z32, lrl}, grid, dim3(TX, TY), 0, s);
         }
     }
+    if constexpr (sizeof(TI) == 8 && MODE != 2) {
+        if (L.n[0] % 2 == 0) {
+            int zc = 0;
+            const int lrl = vw_lrl(L.n[0], 2);
+            const dim3 grid = vw_grid(L, 2, lrl, zc, 16);
+            return launch_k(SweepVK<TI, MODE, 2>{L, ein, r, eout, p, st, zc, z32, lrl}, grid, dim3(TX, TY), 0, s);
+        }
+    }
     // four cells per thread on large grids and in batches (one launch for all cases of a level)
     if (L.N >= (1 << 20) || g_rec)
         return launch_k(SweepK<TI, MODE, 4>{L, ein, r, eout, p, st, z32}, walk_grid(L, 4), dim3(TX, TY), 0, s);
@@ -1904,10 +2072,20 @@ cudaError_t launch_resid_restrict(int inner, const LevelDev& Lf, const LevelDev&
         return launch_k(RRVK<B, 4>{Lf, Lc, (const B*)e, (const B*)r, (B*)rc, (B*)ec0, lrl, st}, grid, dim3(TX, TY), 0,
                         s);
     }
+    if (inner == FVM_FP64 && Lf.active[0] && Lf.active[1]) {   // (active axes of a level that is coarsened are even)
+        const int lrl = vw_lrl(Lf.n[0], 2), wx = 2 << lrl, wy = TY << (5 - lrl);
+        const dim3 grid((unsigned)((Lf.n[0] + wx - 1) / wx), (unsigned)((Lc.n[1] + wy - 1) / wy), (unsigned)Lc.n[2]);
+        return launch_k(RRVK<double, 2>{Lf, Lc, (const double*)e, (const double*)r, (double*)rc, (double*)ec0, lrl, st},
+                        grid, dim3(TX, TY), 0, s);
+    }
     if (Lf.active[0] && Lf.active[1]) {
         const int fz = Lf.active[2] ? 2 : 1;
-        DISPATCH_I(inner, err = launch_k(RRWalkK<TI>{Lf, Lc, (const TI*)e, (const TI*)r, (TI*)rc, (TI*)ec0, st},
-                                         walk_grid(Lf, fz), dim3(TX, TY), 0, s));
+        auto walk = [&](auto ti) {
+            using TI = decltype(ti);
+            return launch_k(RRWalkK<TI>{Lf, Lc, (const TI*)e, (const TI*)r, (TI*)rc, (TI*)ec0, st}, walk_grid(Lf, fz),
+                            dim3(TX, TY), 0, s);
+        };
+        err = inner == FVM_FP32 ? walk(0.0f) : walk(__nv_bfloat16());
     } else {
         DISPATCH_I(inner, err = launch_k(ResidRestrictK<TI>{Lf, Lc, (const TI*)e, (const TI*)r, (TI*)rc, (TI*)ec0,
                                                             st},
@@ -1938,6 +2116,12 @@ cudaError_t launch_prolong_add(int inner, const LevelDev& Lf, const LevelDev& Lc
         const dim3 grid = vw_grid(Lf, 4, lrl, zc);
         return launch_k(ProlongVK<__nv_bfloat16, 4>{Lf, Lc, (const __nv_bfloat16*)ec, (__nv_bfloat16*)e, st, zc, lrl},
                         grid, dim3(TX, TY), 0, s);
+    }
+    if (inner == FVM_FP64 && Lf.active[0] && Lf.active[1]) {
+        int zc = 0;
+        const int lrl = vw_lrl(Lf.n[0], 2);
+        const dim3 grid = vw_grid(Lf, 2, lrl, zc);
+        return launch_k(ProlongVK<double, 2>{Lf, Lc, (const double*)ec, (double*)e, st, zc, lrl}, grid, dim3(TX, TY), 0, s);
     }
     DISPATCH_I(inner, err = launch_k(ProlongK<TI>{Lf, Lc, (const TI*)ec, (TI*)e, st}, grid3(Lf), kBlock3, 0, s));
     return err;
@@ -1971,6 +2155,18 @@ static cudaError_t fcg_launch(const LevelDev& L, const TZ* z, const TR* r, TZ* d
             if (err != cudaSuccess) return err;
             const unsigned nb = (unsigned)((L.N / 4 + FcgUpdVK<TZ, 4>::kThreads - 1) / FcgUpdVK<TZ, 4>::kThreads);
             return launch_k(FcgUpdVK<TZ, 4>{L, z, dp, p, st}, dim3(nb), dim3(FcgUpdVK<TZ, 4>::kThreads), 0, s);
+        }
+    }
+    if constexpr (sizeof(TR) == 8) {
+        if (L.n[0] % 2 == 0) {
+            int zc = 0;
+            const int lrl = vw_lrl(L.n[0], 2);
+            const dim3 grid = vw_grid(L, 2, lrl, zc);
+            cudaError_t err =
+                launch_k(FcgDotVK<TR, TZ, 2>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s);
+            if (err != cudaSuccess) return err;
+            const unsigned nb = (unsigned)((L.N / 2 + FcgUpdVK<TZ, 2>::kThreads - 1) / FcgUpdVK<TZ, 2>::kThreads);
+            return launch_k(FcgUpdVK<TZ, 2>{L, z, dp, p, st}, dim3(nb), dim3(FcgUpdVK<TZ, 2>::kThreads), 0, s);
         }
     }
     cudaError_t err = launch_k(FcgDotK<TR, TZ>{L, z, r, dp, partials, st}, grid3(L), kBlock3, 0, s);
