@@ -163,12 +163,16 @@ struct LevelDev {
     float ih2af[3];
     float ih2alo[3];         // ih2a - ih2af (float-float coefficients)
     int32_t zc_fixed;        // z planes per block of the four-cell kernels (0: the rule)
-    const uint8_t* solid;    // nonzero = solid
-    const uint8_t* dir[6];   // per boundary-face cell: 1 = Dirichlet (p = 0 on the face)
     const uint16_t* nbf;     // per cell: 2 bits per face (x-,x+,y-,y+,z-,z+): 0 fluid neighbour,
                              // 1 zero-gradient ghost, 2 zero-value ghost; bit 12: the cell is solid;
                              // bit 13: a face whose ghost is not the clamped in-grid load (a zero-value
                              // face, or a zero-gradient face towards a solid neighbour)
+    const uint8_t* grp;      // per four cells c, c + 1, .. (c % 4 = 0) four bits, two groups a byte: 1 one of
+                             // them needs its code (solid, a solid neighbour, a zero-value face along y or
+                             // z), 2 / 4 the first cell's x- / the last cell's x+ face is a zero-value
+                             // domain face.  Where 1 is clear every ghost is the load clamped into the
+                             // grid, along x with that sign.
+    int32_t solids, pad;     // the level has solid cells
 };
 
 // Device-side state of one pressure solve: the last residual norms and the
@@ -623,6 +627,7 @@ struct Recorder {
     std::string site;                  // set by the caller before each launch site
     double bytes = 0.0;                // algorithmic bytes of the site (given to its first launch)
     int cases = 1;                     // cases of the batch being recorded
+    bool solids = false;               // some of them have solid cells
 };
 
 extern thread_local Recorder* g_rec;

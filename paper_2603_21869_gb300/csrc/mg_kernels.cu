@@ -542,6 +542,27 @@ template <> __device__ __forceinline__ void codes_w<2>(const uint16_t* f, int c,
     o[0] = v & 0xffffu; o[1] = v >> 16;
 }
 
+// The flags of a thread's W cells (4 or 8) from cell c on (LevelDev::grp): whether their codes are
+// needed, and whether the x ghosts at the two ends are negated.  An eighth of a byte a cell where
+// the codes take two: they are a quarter to a third of the bytes of a BF16 sweep, transfer or
+// prolongation, and a row's end at an outlet no longer sends its warp through the general stencil.
+struct GroupFlags {
+    bool codes, neg_l, neg_r;
+};
+template <int W> __device__ __forceinline__ GroupFlags group_flags(const uint8_t* grp, int c) {
+    const uint32_t b = __ldg(grp + (c >> 3));
+    if constexpr (W == 8) return {(b & 0x11u) != 0u, (b & 0x02u) != 0u, (b & 0x40u) != 0u};
+    const uint32_t n = b >> (c & 4);
+    return {(n & 1u) != 0u, (n & 2u) != 0u, (n & 4u) != 0u};
+}
+// The kernels with more loads in flight per thread (residual, residual and restriction, inner
+// products) have two forms: by the flags, for levels without solid cells, and by the codes.  A
+// second, dependent load for some groups of most warps costs a room more than the bytes: 512 x 256
+// x 128 cells, BF16: residual 104 us with the codes, 109 with the flags; residual and restriction 42
+// and 45; inner products and update 141 and 144 (512 x 128 x 128 FP32 channel: 66 and 59, 30 and
+// 25.5, 80 and 67 us, the other way round).
+static bool by_flags(const LevelDev& L) { return g_rec ? !g_rec->solids : !L.solids; }
+
 // cells per thread of the vector kernels on a level of this storage type
 template <class TI> __device__ __host__ constexpr int vec_w() { return sizeof(TI) == 2 ? 8 : (sizeof(TI) == 4 ? 4 : 2); }
 
@@ -693,7 +714,9 @@ __device__ void SweepVK<TI, MODE, W>::run(const BlockAt& at) const {
         const typename R::T ym = R::load(ein, base + om);
         const typename R::T yp = R::load(ein, base + op);
         const typename R::T rr = R::load(r, base + own);
-        codes_w<W>(nbf, base + own, fs);
+        GroupFlags gf = {true, false, false};
+        if constexpr (sizeof(C) == 8) codes_w<W>(nbf, base + own, fs);
+        else gf = group_flags<W>(L.grp, base + own);
         const C xls = lane == 0 ? to_c<C>(ldg(ein + base + xl)) : (C)0;
         const C xrs = lane == LR - 1 ? to_c<C>(ldg(ein + base + xr)) : (C)0;
         const typename R::T en = R::load(ein, min(k + 2, nz - 1) * sz + own);   // plane after next
@@ -701,7 +724,7 @@ __device__ void SweepVK<TI, MODE, W>::run(const BlockAt& at) const {
             const int fb = (k + 3) * sz + own;
             l2_prefetch(ein + fb);
             l2_prefetch(r + fb);
-            l2_prefetch(nbf + fb);
+            if constexpr (sizeof(C) == 8) l2_prefetch(nbf + fb);
         }
         // (no L1 prefetch of the next plane here, unlike the residual and inner-product kernels:
         // with two planes a block the sweep measured 2 % faster without it)
@@ -710,10 +733,9 @@ __device__ void SweepVK<TI, MODE, W>::run(const BlockAt& at) const {
         if (lane == 0) left = xls;
         if (lane == LR - 1) right = xrs;
         if (last) right = R::get(ec, W - 1);
+        if (gf.neg_l) left = -left;   // (a row's first cell: left is the cell itself)
+        if (gf.neg_r) right = -right;
         C v[W];
-        uint32_t any = 0u;   // solid (bit 12) or irregular (bit 13) anywhere among the W cells
-#pragma unroll
-        for (int t = 0; t < W; ++t) any |= fs[t];
         if constexpr (sizeof(C) == 8) {
 #pragma unroll
             for (int t = 0; t < W; ++t) {
@@ -723,7 +745,7 @@ __device__ void SweepVK<TI, MODE, W>::run(const BlockAt& at) const {
                                     R::get(ep, t), ihx, ihy, ihz, dg);
                 v[t] = is_solid(fs[t]) ? (C)0 : fma(wiD, d, eP);
             }
-        } else if (!(any & 0x3000u)) {
+        } else if (!gf.codes) {
             // every cell fluid, each ghost the clamped in-grid load: the plain stencil
 #pragma unroll
             for (int t = 0; t < W; ++t) {
@@ -735,6 +757,7 @@ __device__ void SweepVK<TI, MODE, W>::run(const BlockAt& at) const {
                 v[t] = fma(wiD, R::get(rr, t) - fma(dg, eP, -s), eP);
             }
         } else {
+            codes_w<W>(nbf, base + own, fs);
 #pragma unroll
             for (int t = 0; t < W; ++t) {
                 const C eP = R::get(ec, t);
@@ -768,12 +791,12 @@ __device__ void SweepVK<TI, MODE, W>::run(const BlockAt& at) const {
 #pragma unroll
                 for (int h = 0; h < W / 2; ++h) {
                     float4 a = pp[h];
-                    if (!is_solid(fs[2 * h])) {
+                    if (!gf.codes || !is_solid(fs[2 * h])) {
                         const float2 x = pp_plus(make_float2(a.x, a.y), v[2 * h]);
                         a.x = x.x;
                         a.y = x.y;
                     }
-                    if (!is_solid(fs[2 * h + 1])) {
+                    if (!gf.codes || !is_solid(fs[2 * h + 1])) {
                         const float2 x = pp_plus(make_float2(a.z, a.w), v[2 * h + 1]);
                         a.z = x.x;
                         a.w = x.y;
@@ -1006,7 +1029,7 @@ __device__ __forceinline__ int resid0_sums(double s0, double s1, double* partial
 
 // r = b - A p (float-float), r^2 and b^2, the first pre-sweep e = w_J r / D;
 // four x cells per thread and a z march (the sweep's layout).  FP32 b, nx % 4 = 0.
-template <class TI>
+template <class TI, bool F>   // F: by the group flags
 struct Resid0V4K {
     static constexpr int kThreads = TX * TY;
     static constexpr int kMinBlocks = 3;       // at most 80 registers
@@ -1026,8 +1049,8 @@ struct Resid0V4K {
     __device__ int run(const BlockAt& at) const;
 };
 
-template <class TI>
-__device__ int Resid0V4K<TI>::run(const BlockAt& at) const {
+template <class TI, bool F>
+__device__ int Resid0V4K<TI, F>::run(const BlockAt& at) const {
     const int nx = L.n[0], ny = L.n[1], nz = L.n[2];
     const int LR = 1 << lrl, lane = threadIdx.x & (LR - 1), sub = threadIdx.x >> lrl;
     const int i4 = at.b.x * (4 * LR) + lane * 4, j = ((at.b.y * TY + threadIdx.y) << (5 - lrl)) + sub;
@@ -1055,7 +1078,10 @@ __device__ int Resid0V4K<TI>::run(const BlockAt& at) const {
         ff_load4(pp, base + om, ym);
         ff_load4(pp, base + op, yp);
         const float4 bq = __ldg(reinterpret_cast<const float4*>(b + base + own));
-        const uint2 fw = __ldg(reinterpret_cast<const uint2*>(nbf + base + own));
+        GroupFlags gf = {true, false, false};
+        if constexpr (F) gf = group_flags<4>(L.grp, base + own);
+        uint32_t fs[4] = {0u, 0u, 0u, 0u};
+        if (gf.codes) codes_w<4>(nbf, base + own, fs);
         const FF xls = lane == 0 ? pp_load(pp, base + xl) : FF{0.0f, 0.0f};
         const FF xrs = lane == LR - 1 ? pp_load(pp, base + xr) : FF{0.0f, 0.0f};
         ff_load4(pp, min(k + 2, nz - 1) * sz + own, en);
@@ -1064,22 +1090,25 @@ __device__ int Resid0V4K<TI>::run(const BlockAt& at) const {
             l2_prefetch(pp + fb);
             l2_prefetch(pp + fb + 2);
             l2_prefetch(b + fb);
-            l2_prefetch(nbf + fb);
+            if constexpr (!F) l2_prefetch(nbf + fb);
         }
         if (k + 1 < k1) {   // the next plane's rows into L1 (their loads open the next iteration)
             const int nb = (k + 1) * sz;
             l1_prefetch(pp + nb + om);
             l1_prefetch(pp + nb + op);
             l1_prefetch(b + nb + own);
-            l1_prefetch(nbf + nb + own);
+            if constexpr (!F) l1_prefetch(nbf + nb + own);
         }
         FF left = {__shfl_up_sync(0xffffffffu, ec[3].h, 1, LR), __shfl_up_sync(0xffffffffu, ec[3].l, 1, LR)};
         FF right = {__shfl_down_sync(0xffffffffu, ec[0].h, 1, LR), __shfl_down_sync(0xffffffffu, ec[0].l, 1, LR)};
         if (lane == 0) left = xls;
         if (lane == LR - 1) right = xrs;
         if (lastc) right = ec[3];
+        if constexpr (F) {   // (at a row's ends left / right is the cell itself)
+            if (gf.neg_l) left = ff_neg(left);
+            if (gf.neg_r) right = ff_neg(right);
+        }
         const FF xs[6] = {left, ec[0], ec[1], ec[2], ec[3], right};
-        const uint32_t fs[4] = {fw.x & 0xffffu, fw.x >> 16, fw.y & 0xffffu, fw.y >> 16};
         const float bb[4] = {bq.x, bq.y, bq.z, bq.w};
         // b - A p: a pair of regular cells (code bit 13 clear) in the packed form, any other cell alone
         float rfs[4];
@@ -1106,9 +1135,8 @@ __device__ int Resid0V4K<TI>::run(const BlockAt& at) const {
         float rv[4], ev[4];
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
-            const uint32_t f = fs[t];
             const float rf = rfs[t];
-            const bool fluid = !is_solid(f);
+            const bool fluid = !is_solid(fs[t]);
             const float rc = fluid ? round_inner<TI>(rf) : 0.0f;
             rv[t] = rc;
             ev[t] = wJ * rc * iD;
@@ -1191,7 +1219,7 @@ __device__ int Resid0D2K::run(const BlockAt& at) const {
 // (the sweep's layout and neighbour scheme): products, the thread's and the
 // warp's sums in FP32, block and grid sums in FP64.  Needs nx % W = 0.
 // (TR: storage of r; TZ: storage of z and the kept direction, FP32 on BF16 levels)
-template <class TR, class TZ, int W>
+template <class TR, class TZ, int W, bool F>   // F: by the group flags
 struct FcgDotVK {
     static constexpr int kThreads = TX * TY;
     static constexpr int kMinBlocks = 4;       // at most 64 registers
@@ -1208,8 +1236,8 @@ struct FcgDotVK {
     __device__ void run(const BlockAt& at) const;
 };
 
-template <class TR, class TZ, int W>
-__device__ void FcgDotVK<TR, TZ, W>::run(const BlockAt& at) const {
+template <class TR, class TZ, int W, bool F>
+__device__ void FcgDotVK<TR, TZ, W, F>::run(const BlockAt& at) const {
     using C = typename Acc<TZ>::type;
     using R = RawW<TZ, W>;
     using RR = RawW<TR, W>;
@@ -1240,7 +1268,9 @@ __device__ void FcgDotVK<TR, TZ, W>::run(const BlockAt& at) const {
         typename R::T dd = {};
         if (have) dd = R::load(dp, base + own);
         uint32_t fs[W];
-        codes_w<W>(nbf, base + own, fs);
+        GroupFlags gf = {true, false, false};
+        if constexpr (F) gf = group_flags<W>(L.grp, base + own);
+        if (gf.codes) codes_w<W>(nbf, base + own, fs);
         const C xls = lane == 0 ? to_c<C>(ldg(zz + base + xl)) : (C)0;
         const C xrs = lane == LR - 1 ? to_c<C>(ldg(zz + base + xr)) : (C)0;
         const typename R::T en = R::load(zz, min(k + 2, nz - 1) * sz + own);
@@ -1248,7 +1278,7 @@ __device__ void FcgDotVK<TR, TZ, W>::run(const BlockAt& at) const {
             const int fb = (k + 3) * sz + own;
             l2_prefetch(zz + fb);
             l2_prefetch(r + fb);
-            l2_prefetch(nbf + fb);
+            if constexpr (!F) l2_prefetch(nbf + fb);
             if (have) l2_prefetch(dp + fb);
         }
         if (k + 1 < k1) {   // the next plane's rows into L1 (their loads open the next iteration)
@@ -1256,7 +1286,7 @@ __device__ void FcgDotVK<TR, TZ, W>::run(const BlockAt& at) const {
             l1_prefetch(zz + nb + om);
             l1_prefetch(zz + nb + op);
             l1_prefetch(r + nb + own);
-            l1_prefetch(nbf + nb + own);
+            if constexpr (!F) l1_prefetch(nbf + nb + own);
             if (have) l1_prefetch(dp + nb + own);
         }
         C left = __shfl_up_sync(0xffffffffu, R::get(ec, W - 1), 1, LR);
@@ -1264,13 +1294,19 @@ __device__ void FcgDotVK<TR, TZ, W>::run(const BlockAt& at) const {
         if (lane == 0) left = xls;
         if (lane == LR - 1) right = xrs;
         if (lastc) right = R::get(ec, W - 1);
-        uint32_t any = 0u;   // solid (bit 12) or irregular (bit 13) anywhere among the W cells
+        if constexpr (F) {   // (at a row's ends left / right is the cell itself)
+            if (gf.neg_l) left = -left;
+            if (gf.neg_r) right = -right;
+        } else {
+            uint32_t any = 0u;   // solid (bit 12) or irregular (bit 13) anywhere among the W cells
 #pragma unroll
-        for (int t = 0; t < W; ++t) any |= fs[t];
+            for (int t = 0; t < W; ++t) any |= fs[t];
+            gf.codes = (any & 0x3000u) != 0u;
+        }
         if (in) {
 #pragma unroll
             for (int t = 0; t < W; ++t) {
-                const bool plain = !(any & 0x3000u);   // every cell fluid with in-grid ghosts
+                const bool plain = !gf.codes;   // every cell fluid with in-grid ghosts
                 if (!plain && is_solid(fs[t])) continue;
                 const C eP = R::get(ec, t);
                 const C xm = t == 0 ? left : R::get(ec, t - 1), xp = t == W - 1 ? right : R::get(ec, t + 1);
@@ -1324,7 +1360,10 @@ struct FcgUpdVK {
         VecW<TZ, W>::load(z, c, zv);
         if (beta != (C)0) VecW<TZ, W>::load_rw(dp, c, dv);
         uint32_t fs[W];
-        codes_w<W>(L.nbf, c, fs);
+        GroupFlags gf = {true, false, false};
+        if constexpr (sizeof(C) == 4) gf = group_flags<W>(L.grp, c);
+        const bool codes = gf.codes;
+        if (codes) codes_w<W>(L.nbf, c, fs);
         C d[W];
 #pragma unroll
         for (int t = 0; t < W; ++t) d[t] = fma(-beta, dv[t], zv[t]);
@@ -1342,12 +1381,12 @@ struct FcgUpdVK {
 #pragma unroll
         for (int h = 0; h < W / 2; ++h) {
             float4 u = pp[h];
-            if (!is_solid(fs[2 * h])) {
+            if (!codes || !is_solid(fs[2 * h])) {
                 const float2 x = pp_plus(make_float2(u.x, u.y), alpha * d[2 * h]);
                 u.x = x.x;
                 u.y = x.y;
             }
-            if (!is_solid(fs[2 * h + 1])) {
+            if (!codes || !is_solid(fs[2 * h + 1])) {
                 const float2 x = pp_plus(make_float2(u.z, u.w), alpha * d[2 * h + 1]);
                 u.z = x.x;
                 u.w = x.y;
@@ -1472,10 +1511,13 @@ __device__ void ProlongVK<TI, W>::run(const BlockAt& at) const {
             C v[W];
             uint32_t fs[W];
             VecW<TI, W>::load_rw(ep, c, v);
-            codes_w<W>(nbf, c, fs);
+            GroupFlags gf = {true, false, false};
+            if constexpr (sizeof(C) == 4) gf = group_flags<W>(Lf.grp, c);
+            const bool codes = gf.codes;
+            if (codes) codes_w<W>(nbf, c, fs);
 #pragma unroll
             for (int t = 0; t < W; ++t)
-                if (!is_solid(fs[t])) v[t] += add[t];
+                if (!codes || !is_solid(fs[t])) v[t] += add[t];
             VecW<TI, W>::store(ep, c, v);
         }
     }
@@ -1486,7 +1528,7 @@ __device__ void ProlongVK<TI, W>::run(const BlockAt& at) const {
 // writes the W/2 coarse cells I0 = i4/2 .. (mean of their children's r - A e,
 // Eq. restriction).  Rows j +- 1 and planes k +- 1 are loaded whole, x
 // neighbours by shuffles.  Needs x and y active, nx % W = 0, ny even.
-template <class TI, int W>
+template <class TI, int W, bool F>   // F: by the group flags
 struct RRVK {
     static constexpr int kThreads = TX * TY;
     static constexpr bool kNoShared = true;   // run() uses no shared memory
@@ -1502,8 +1544,8 @@ struct RRVK {
     __device__ void run(const BlockAt& at) const;
 };
 
-template <class TI, int W>
-__device__ void RRVK<TI, W>::run(const BlockAt& at) const {
+template <class TI, int W, bool F>
+__device__ void RRVK<TI, W, F>::run(const BlockAt& at) const {
     using C = typename Acc<TI>::type;
     using R = RawW<TI, W>;
     constexpr int H = W / 2;
@@ -1539,7 +1581,9 @@ __device__ void RRVK<TI, W>::run(const BlockAt& at) const {
             const typename R::T zh = R::load(ep, at_(jr, kp));
             const typename R::T rr = R::load(rp, at_(jr, k));
             uint32_t fs[W];
-            codes_w<W>(nbf, at_(jr, k), fs);
+            GroupFlags gf = {true, false, false};
+            if constexpr (F) gf = group_flags<W>(Lf.grp, at_(jr, k));
+            if (gf.codes) codes_w<W>(nbf, at_(jr, k), fs);
             const C lx = lane == 0 ? to_c<C>(ldg(ep + max(ic - 1, 0) + sy * jr + sz * k)) : (C)0;
             const C rx = lane == LR - 1 ? to_c<C>(ldg(ep + min(ic + W, nx - 1) + sy * jr + sz * k)) : (C)0;
             C left = __shfl_up_sync(0xffffffffu, R::get(ec, W - 1), 1, LR);
@@ -1547,9 +1591,13 @@ __device__ void RRVK<TI, W>::run(const BlockAt& at) const {
             if (lane == 0) left = lx;
             if (lane == LR - 1) right = rx;
             if (last) right = R::get(ec, W - 1);
+            if constexpr (F) {   // (at a row's ends left / right is the cell itself)
+                if (gf.neg_l) left = -left;
+                if (gf.neg_r) right = -right;
+            }
 #pragma unroll
             for (int t = 0; t < W; ++t) {
-                if (is_solid(fs[t])) continue;
+                if ((!F || gf.codes) && is_solid(fs[t])) continue;
                 const C eP = R::get(ec, t);
                 const C xm = t == 0 ? left : R::get(ec, t - 1), xp = t == W - 1 ? right : R::get(ec, t + 1);
                 const C ya = R::get(yl, t), yb = R::get(yh, t), za = R::get(zl, t), zb = R::get(zh, t);
@@ -1558,7 +1606,7 @@ __device__ void RRVK<TI, W>::run(const BlockAt& at) const {
                     continue;
                 }
                 C A;
-                if (!((fs[t] >> 13) & 1u)) {
+                if ((F && !gf.codes) || !((fs[t] >> 13) & 1u)) {
                     C sa = (xm + xp) * ihx;
                     sa = fma(ya + yb, ihy, sa);
                     sa = fma(za + zb, ihz, sa);
@@ -1923,7 +1971,10 @@ cudaError_t launch_resid0(int inner, int bprec, const LevelDev& L, const double*
                 int zc = 0;
                 const dim3 grid = v4_grid(L, lrl, zc);
                 // (at most level0_blocks_max(n) blocks: partials has room)
-                return launch_r0(Resid0V4K<TI>{L, p, (const float*)b, (TI*)r, (TI*)e, partials, st, zc, lrl}, grid,
+                if (by_flags(L))
+                    return launch_r0(Resid0V4K<TI, true>{L, p, (const float*)b, (TI*)r, (TI*)e, partials, st, zc, lrl},
+                                     grid, dim3(TX, TY), cond, use_cond, s);
+                return launch_r0(Resid0V4K<TI, false>{L, p, (const float*)b, (TI*)r, (TI*)e, partials, st, zc, lrl}, grid,
                                  dim3(TX, TY), cond, use_cond, s);
             }
         }
@@ -2062,20 +2113,26 @@ cudaError_t launch_resid_restrict(int inner, const LevelDev& Lf, const LevelDev&
         const int W = inner == FVM_BF16_MIXED && wide8(Lf) ? 8 : 4;
         const int lrl = vw_lrl(Lf.n[0], W), wx = W << lrl, wy = TY << (5 - lrl);
         const dim3 grid((unsigned)((Lf.n[0] + wx - 1) / wx), (unsigned)((Lc.n[1] + wy - 1) / wy), (unsigned)Lc.n[2]);
-        if (inner == FVM_FP32)
-            return launch_k(RRVK<float, 4>{Lf, Lc, (const float*)e, (const float*)r, (float*)rc, (float*)ec0, lrl, st},
+        auto go = [&](auto ti, auto w, auto f) {
+            using TI = decltype(ti);
+            return launch_k(RRVK<TI, decltype(w)::value, decltype(f)::value>{Lf, Lc, (const TI*)e, (const TI*)r, (TI*)rc,
+                                                                             (TI*)ec0, lrl, st},
                             grid, dim3(TX, TY), 0, s);
-        using B = __nv_bfloat16;
-        if (W == 8)
-            return launch_k(RRVK<B, 8>{Lf, Lc, (const B*)e, (const B*)r, (B*)rc, (B*)ec0, lrl, st}, grid, dim3(TX, TY),
-                            0, s);
-        return launch_k(RRVK<B, 4>{Lf, Lc, (const B*)e, (const B*)r, (B*)rc, (B*)ec0, lrl, st}, grid, dim3(TX, TY), 0,
-                        s);
+        };
+        using W4 = std::integral_constant<int, 4>;
+        using W8 = std::integral_constant<int, 8>;
+        using Yes = std::true_type;
+        using No = std::false_type;
+        const bool f = by_flags(Lf);
+        if (inner == FVM_FP32) return f ? go(0.0f, W4(), Yes()) : go(0.0f, W4(), No());
+        const __nv_bfloat16 b16{};
+        if (W == 8) return f ? go(b16, W8(), Yes()) : go(b16, W8(), No());
+        return f ? go(b16, W4(), Yes()) : go(b16, W4(), No());
     }
     if (inner == FVM_FP64 && Lf.active[0] && Lf.active[1]) {   // (active axes of a level that is coarsened are even)
         const int lrl = vw_lrl(Lf.n[0], 2), wx = 2 << lrl, wy = TY << (5 - lrl);
         const dim3 grid((unsigned)((Lf.n[0] + wx - 1) / wx), (unsigned)((Lc.n[1] + wy - 1) / wy), (unsigned)Lc.n[2]);
-        return launch_k(RRVK<double, 2>{Lf, Lc, (const double*)e, (const double*)r, (double*)rc, (double*)ec0, lrl, st},
+        return launch_k(RRVK<double, 2, false>{Lf, Lc, (const double*)e, (const double*)r, (double*)rc, (double*)ec0, lrl, st},
                         grid, dim3(TX, TY), 0, s);
     }
     if (Lf.active[0] && Lf.active[1]) {
@@ -2143,7 +2200,8 @@ static cudaError_t fcg_launch(const LevelDev& L, const TZ* z, const TR* r, TZ* d
                 const int lrl = vw_lrl(L.n[0], W);
                 const dim3 grid = vw_grid(L, W, lrl, zc);
                 cudaError_t err =
-                    launch_k(FcgDotVK<TR, TZ, W>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s);
+                    by_flags(L) ? launch_k(FcgDotVK<TR, TZ, W, true>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s)
+                                : launch_k(FcgDotVK<TR, TZ, W, false>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s);
                 if (err != cudaSuccess) return err;
                 const unsigned nb = (unsigned)((L.N / W + FcgUpdVK<TZ, W>::kThreads - 1) / FcgUpdVK<TZ, W>::kThreads);
                 return launch_k(FcgUpdVK<TZ, W>{L, z, dp, p, st}, dim3(nb), dim3(FcgUpdVK<TZ, W>::kThreads), 0, s);
@@ -2151,7 +2209,8 @@ static cudaError_t fcg_launch(const LevelDev& L, const TZ* z, const TR* r, TZ* d
             const int lrl = vw_lrl(L.n[0], 4);
             const dim3 grid = vw_grid(L, 4, lrl, zc);
             cudaError_t err =
-                launch_k(FcgDotVK<TR, TZ, 4>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s);
+                by_flags(L) ? launch_k(FcgDotVK<TR, TZ, 4, true>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s)
+                            : launch_k(FcgDotVK<TR, TZ, 4, false>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s);
             if (err != cudaSuccess) return err;
             const unsigned nb = (unsigned)((L.N / 4 + FcgUpdVK<TZ, 4>::kThreads - 1) / FcgUpdVK<TZ, 4>::kThreads);
             return launch_k(FcgUpdVK<TZ, 4>{L, z, dp, p, st}, dim3(nb), dim3(FcgUpdVK<TZ, 4>::kThreads), 0, s);
@@ -2163,7 +2222,7 @@ static cudaError_t fcg_launch(const LevelDev& L, const TZ* z, const TR* r, TZ* d
             const int lrl = vw_lrl(L.n[0], 2);
             const dim3 grid = vw_grid(L, 2, lrl, zc);
             cudaError_t err =
-                launch_k(FcgDotVK<TR, TZ, 2>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s);
+                launch_k(FcgDotVK<TR, TZ, 2, false>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s);
             if (err != cudaSuccess) return err;
             const unsigned nb = (unsigned)((L.N / 2 + FcgUpdVK<TZ, 2>::kThreads - 1) / FcgUpdVK<TZ, 2>::kThreads);
             return launch_k(FcgUpdVK<TZ, 2>{L, z, dp, p, st}, dim3(nb), dim3(FcgUpdVK<TZ, 2>::kThreads), 0, s);

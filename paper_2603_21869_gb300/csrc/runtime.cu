@@ -51,40 +51,73 @@ struct HostLevel {
     std::vector<uint8_t> solid;
     std::vector<uint8_t> dir[6];
     std::vector<uint16_t> nbf;
+    std::vector<uint8_t> grp;
+    bool solids = false;
     int64_t N() const { return (int64_t)n[0] * n[1] * n[2]; }
 };
 
-// Neighbour codes of every cell (see LevelDev::nbf).
+// Neighbour codes of every cell and the flags of its group of four (see LevelDev::nbf, grp).  In a
+// row whose own and four neighbouring rows hold no solid cell and lie in the grid only the two end
+// cells have a face: the rest keeps code 0.
 void build_nbf(HostLevel& L) {
+    const int nx = L.n[0], ny = L.n[1], nz = L.n[2];
     L.nbf.assign(L.N(), 0);
-    for (int k = 0; k < L.n[2]; ++k)
-        for (int j = 0; j < L.n[1]; ++j)
-            for (int i = 0; i < L.n[0]; ++i) {
-                const int64_t c = cell_index(i, j, k, L.n[0], L.n[1]);
-                if (L.solid[c]) {
-                    L.nbf[c] = (uint16_t)(1u << 12);
-                    continue;
-                }
-                uint32_t code = 0;
-                bool irregular = false;   // a ghost that a neighbour load clamped into the grid does not give
-                const int f[3] = {i, j, k};
-                for (int d = 0; d < 6; ++d) {
-                    const int a = d / 2, side = (d & 1) ? 1 : -1;
-                    int q[3] = {f[0], f[1], f[2]};
-                    q[a] += side;
-                    uint32_t v;
-                    if (q[a] < 0 || q[a] >= L.n[a]) {
-                        v = L.dir[d][face_index(a, i, j, k, L.n)] ? 2u : 1u;
-                        irregular = irregular || v == 2u;
-                    } else {
-                        v = L.solid[cell_index(q[0], q[1], q[2], L.n[0], L.n[1])] ? 1u : 0u;
-                        irregular = irregular || v == 1u;
-                    }
-                    code |= v << (2 * d);
-                }
-                if (irregular) code |= 1u << 13;
-                L.nbf[c] = (uint16_t)code;
+    L.grp.assign((size_t)((L.N() + 7) / 8), 0);
+    std::vector<uint8_t> row_solid((size_t)ny * nz);
+    L.solids = false;
+    for (size_t r = 0; r < row_solid.size(); ++r) {
+        row_solid[r] = memchr(L.solid.data() + r * nx, 1, (size_t)nx) != nullptr;
+        L.solids = L.solids || row_solid[r];
+    }
+    uint8_t* const grp = L.grp.data();
+    auto flag = [&](int64_t c, uint32_t f) { grp[c >> 3] |= (uint8_t)(f << (4 * ((c >> 2) & 1))); };
+    auto cell = [&](int i, int j, int k) {
+        const int64_t c = cell_index(i, j, k, nx, ny);
+        if (L.solid[c]) {
+            L.nbf[c] = (uint16_t)(1u << 12);
+            flag(c, 1u);
+            return;
+        }
+        uint32_t code = 0;
+        bool irregular = false;   // a ghost that a neighbour load clamped into the grid does not give
+        const int f[3] = {i, j, k};
+        for (int d = 0; d < 6; ++d) {
+            const int a = d / 2, side = (d & 1) ? 1 : -1;
+            int q[3] = {f[0], f[1], f[2]};
+            q[a] += side;
+            uint32_t v;
+            if (q[a] < 0 || q[a] >= L.n[a]) {
+                v = L.dir[d][face_index(a, i, j, k, L.n)] ? 2u : 1u;
+                irregular = irregular || v == 2u;
+                if (v == 2u) flag(c, a > 0 ? 1u : (side < 0 ? 2u : 4u));
+            } else {
+                v = L.solid[cell_index(q[0], q[1], q[2], nx, ny)] ? 1u : 0u;
+                irregular = irregular || v == 1u;
+                if (v == 1u) flag(c, 1u);
             }
+            code |= v << (2 * d);
+        }
+        if (irregular) code |= 1u << 13;
+        L.nbf[c] = (uint16_t)code;
+    };
+    for (int k = 0; k < nz; ++k)
+        for (int j = 0; j < ny; ++j) {
+            const size_t r = (size_t)k * ny + j;
+            const bool inner = j > 0 && j < ny - 1 && k > 0 && k < nz - 1;
+            if (inner && !row_solid[r] && !row_solid[r - 1] && !row_solid[r + 1] && !row_solid[r - ny] && !row_solid[r + ny]) {
+                cell(0, j, k);
+                if (nx > 1) cell(nx - 1, j, k);
+            } else {
+                const uint8_t* const q = L.solid.data() + r * nx;
+                const int64_t sz = (int64_t)nx * ny;
+                for (int i = 0; i < nx; ++i) {
+                    if (inner && i > 0 && i < nx - 1 &&
+                        !(q[i] | q[i - 1] | q[i + 1] | q[i - nx] | q[i + nx] | q[i - sz] | q[i + sz]))
+                        continue;
+                    cell(i, j, k);
+                }
+            }
+        }
 }
 
 int face_cells(const int* n, int face) {
@@ -551,8 +584,7 @@ fvm_status plan_case(const fvm_case_desc* d, Plan& pl) {
     for (int f = 0; f < 6; ++f) bytes += face_cells(n, f);
     for (size_t l = 0; l < pl.levels.size(); ++l) {
         const int64_t NL = pl.levels[l].N();
-        bytes += 3 * NL * si + (l ? NL : 0) + 2 * NL;
-        for (int f = 0; f < 6; ++f) bytes += l ? (int64_t)pl.levels[l].dir[f].size() : 0;
+        bytes += 3 * NL * si + 2 * NL + (NL + 7) / 8;
     }
     const int64_t nc = pl.levels.back().N();
     bytes += nc * nc * 12;   // coarsest inverse, FP64 and FP32
@@ -1240,23 +1272,15 @@ fvm_status build_case(const Plan& pl, fvm_case* c) {
         v.wJf = (float)v.wJ;
         v.diagf = (float)v.diag;
         v.zc_fixed = d.sweep_planes;
-        if (l == 0) v.solid = tag_d;
-        else {
-            uint8_t* sd;
-            ST_TRY(dalloc(c, (void**)&sd, v.N));
-            CUDA_TRY(cudaMemcpyAsync(sd, H.solid.data(), v.N, cudaMemcpyHostToDevice, c->stream));
-            v.solid = sd;
-        }
-        for (int f = 0; f < 6; ++f) {
-            uint8_t* dd;
-            ST_TRY(dalloc(c, (void**)&dd, H.dir[f].size()));
-            CUDA_TRY(cudaMemcpyAsync(dd, H.dir[f].data(), H.dir[f].size(), cudaMemcpyHostToDevice, c->stream));
-            v.dir[f] = dd;
-        }
         uint16_t* nb;
         ST_TRY(dalloc(c, (void**)&nb, v.N * 2));
         CUDA_TRY(cudaMemcpyAsync(nb, H.nbf.data(), v.N * 2, cudaMemcpyHostToDevice, c->stream));
         v.nbf = nb;
+        uint8_t* gr;
+        ST_TRY(dalloc(c, (void**)&gr, H.grp.size()));
+        CUDA_TRY(cudaMemcpyAsync(gr, H.grp.data(), H.grp.size(), cudaMemcpyHostToDevice, c->stream));
+        v.grp = gr;
+        v.solids = H.solids;
         if (l == 0) {
             cd.nbf0 = nb;
             cd.regular_mask = (H.active[0] ? 0x00fu : 0u) | (H.active[1] ? 0x0f0u : 0u) | (H.active[2] ? 0xf00u : 0u) |
@@ -1635,6 +1659,7 @@ fvm_status batch_capture(fvm_batch* B, fvm_batch::Graph& G) {
         }
         Recorder R;
         R.cases = n;
+        for (const fvm_case* q : B->cases) R.solids = R.solids || q->levels[0].dev.solids;
         g_rec = &R;
         for (int k : kStepStages)
             if (st == FVM_OK) st = stage(c, k, nullptr, nullptr);
