@@ -460,19 +460,22 @@ __device__ __forceinline__ void face_flux(const CaseDev& cd, int a, const St<C>&
     fl[a] -= (C)(2.0 / 3.0) * ((C)0.5 * (L.k + R.k));
 }
 
-// face nu_t: 0 on walls, the mean of the two cells inside, the cell's own on other faces
-template <class C, class N>
-__device__ __forceinline__ C face_nut(int kind, C nutP, N nut_nb) {
-    if (kind == FK_WALL) return (C)0;
-    if (kind == FK_INTERIOR) return (C)0.5 * (nutP + nut_nb());
-    return nutP;
-}
+// (nu_t on a face: 0 on walls, the mean of the two cells inside, the cell's own on other faces)
 
+// Each face between two fluid cells is computed once and used by both: along x by the upper cell's
+// lane, which hands its flux down by a shuffle (a warp owns 31 cells of a row, its last lane only the
+// face above them), along y by the upper row, through shared memory (a block is eight rows; the
+// topmost computes its own upper face), along z by a march of zc planes, carried in registers.  Only
+// a face towards a boundary or a solid cell belongs to one cell, which forms its ghost.
+// FP32 is bound by the issue of the flux arithmetic and its loads, FP64 by the FP64 pipe (a 64th of
+// the FP32 rate); a thread a cell computed every inner face twice.  One cell a thread -> this, us a
+// launch: FP32 256 x 64 x 64 36.8 -> 33.7, 512 x 128 x 128 266 -> 203, BF16-mixed room
+// 512 x 256 x 128 522 -> 389, eight FP32 channels of 256 x 64 x 64 in a batch 277 -> 208; FP64
+// 256 x 64 x 64 770 -> 718 (at 128 registers; 747 with one block an SM and no spills).
 template <class S, class C, bool kBlend>
 struct ExplicitK {
-    static constexpr int kThreads = BX * BY * BZ;
-    static constexpr bool kNoShared = true;   // run() uses no shared memory
-    static constexpr int kMinBlocks = sizeof(C) == 4 ? 4 : 1;   // FP32: at most 64 registers
+    static constexpr int kThreads = 256, kRows = 8, kCells = 31;
+    static constexpr int kMinBlocks = sizeof(C) == 4 ? 3 : 2;   // FP32: at most 85 registers, FP64: 128
     __device__ bool live() const { return true; }
     CaseDev cd;
     StatePtrs in, out;
@@ -485,8 +488,8 @@ struct ExplicitK {
     StatePtrs base;
     double wb, ws;
     float wbf, wsf;
+    int zc, pad;    // planes per block
     __device__ void run(const BlockAt& at) const;
-    __device__ void cell(int i, int j, int k) const;
 };
 
 // The cell update of the explicit stage from the summed face fluxes rhs (Algorithm 2): the
@@ -515,80 +518,166 @@ __device__ __forceinline__ void exp_update(const CaseDev& cd, const St<C>& P, C 
     o[5] = on > (C)kOmegaMin ? on : (C)kOmegaMin;
 }
 
-template <class S, class C, bool kBlend>
-__device__ void ExplicitK<S, C, kBlend>::run(const BlockAt& at) const {
-    int i, j, k;
-    if (cell3(cd, at, i, j, k)) cell(i, j, k);
+// one face as its cells use it: the flux of the six fields and the velocity differences across it
+template <class C>
+struct Face {
+    C fl[6], d[3];
+};
+
+// the face between the states L (lower) and R (upper) along axis A, nu_t on it nf
+template <int A, class C>
+__device__ __forceinline__ void face_of(const CaseDev& cd, const St<C>& L, const St<C>& R, C nf, Face<C>& F) {
+    face_flux(cd, A, L, R, nf, F.fl);
+    F.d[0] = R.u - L.u;
+    F.d[1] = R.v - L.v;
+    F.d[2] = R.w - L.w;
+}
+
+// a face of the fluid cell (i, j, k) towards a boundary or a solid cell; returns whether it is a wall
+template <int A, int Side, class S, class C>
+__device__ __forceinline__ bool ghost_face(const CaseDev& cd, const StatePtrs& st, int i, int j, int k, const St<C>& P,
+                                           C nutP, Face<C>& F) {
+    St<C> g;
+    const bool wall = neighbour<S, C>(cd, st, i, j, k, A, Side, P, g) == FK_WALL;
+    const C nf = wall ? (C)0 : nutP;
+    if (Side < 0) face_of<A>(cd, g, P, nf, F);
+    else face_of<A>(cd, P, g, nf, F);
+    return wall;
+}
+
+// the two faces of axis A into the cell's right-hand side and velocity gradient
+template <int A, class C>
+__device__ __forceinline__ void add_axis(const CaseDev& cd, const Face<C>& lo, const Face<C>& hi, C rhs[6], C gu[3][3]) {
+    const C ih = prm<C>(cd.inv_h[A], cd.f.inv_h[A]);
+#pragma unroll
+    for (int f = 0; f < 6; ++f) rhs[f] += (hi.fl[f] - lo.fl[f]) * ih;
+#pragma unroll
+    for (int v = 0; v < 3; ++v) gu[v][A] = (C)0.5 * (hi.d[v] * ih + lo.d[v] * ih);
 }
 
 template <class S, class C, bool kBlend>
-__device__ void ExplicitK<S, C, kBlend>::cell(int i, int j, int k) const {
-    const int c = i + cd.n[0] * (j + cd.n[1] * k);
-    const St<C> P = load_state<S, C>(in, c);
-    S* o[6];
-    for (int f = 0; f < 6; ++f) o[f] = (S*)out.f[f];
-    if (cd.tag[c]) {
-        o[0][c] = from_c<S, C>(P.u); o[1][c] = from_c<S, C>(P.v); o[2][c] = from_c<S, C>(P.w);
-        o[3][c] = from_c<S, C>(P.T); o[4][c] = from_c<S, C>(P.k); o[5][c] = from_c<S, C>(P.om);
-        return;
-    }
-    const C nu = prm<C>(cd.nu, cd.f.nu);
+__device__ void ExplicitK<S, C, kBlend>::run(const BlockAt& at) const {
+    __shared__ C rows[2][9][kRows][32];   // the lower y faces of the block's rows, this plane's and the last one's
+    const int nx = cd.n[0], ny = cd.n[1], nz = cd.n[2];
+    const int lane = threadIdx.x, row = threadIdx.y;
+    const int nrows = blockDim.y;
+    const int i = (int)at.b.x * kCells + lane, j = (int)at.b.y * nrows + row;
+    const int k0 = (int)at.b.z * zc, k1 = min(nz, k0 + zc);
+    const int ic = min(i, nx - 1), jc = min(j, ny - 1);
+    const bool own = lane < kCells && i < nx && j < ny;
+    const int sy = nx, sz = nx * ny;
+    const C nu = prm<C>(cd.nu, cd.f.nu), dt = dt_of<C>(dt_state, 0);
     const S* const nutf = nut;
-    const C nutP = nutf ? to_c<C>(ldg(nutf + c)) : nut_of(P.k, P.om, nu);
-    const int stride[3] = {1, cd.n[0], cd.n[0] * cd.n[1]};
-    const bool reg = regular_cell(cd, c);
-    C rhs[6] = {(C)0, (C)0, (C)0, (C)0, (C)0, (C)0};
-    C gu[3][3];
-    C omw = (C)0;
-    for (int a = 0; a < 3; ++a) {
-        if (!cd.active[a]) {
-            gu[0][a] = gu[1][a] = gu[2][a] = (C)0;
-            continue;
-        }
-        St<C> L, R;
-        int kl = FK_INTERIOR, kr = FK_INTERIOR;
-        if (reg) {
-            L = regular_neighbour<S, C>(cd, in, i, j, k, a, -1);
-            R = regular_neighbour<S, C>(cd, in, i, j, k, a, +1);
-        } else {
-            kl = neighbour<S, C>(cd, in, i, j, k, a, -1, P, L);
-            kr = neighbour<S, C>(cd, in, i, j, k, a, +1, P, R);
-        }
-        C fw[6], fe[6];
-        // (an interior face's neighbour index, its coordinate clamped into the grid like every load)
-        const int q = a == 0 ? i : (a == 1 ? j : k);
-        const int cm = c - (q > 0 ? stride[a] : 0), cp = c + (q < cd.n[a] - 1 ? stride[a] : 0);
-        auto nb_nut = [&](int side, const St<C>& g) {
-            return [&, side]() { return nutf ? to_c<C>(ldg(nutf + (side < 0 ? cm : cp))) : nut_of(g.k, g.om, nu); };
-        };
-        face_flux(cd, a, L, P, face_nut<C>(kl, nutP, nb_nut(-1, L)), fw);
-        face_flux(cd, a, P, R, face_nut<C>(kr, nutP, nb_nut(+1, R)), fe);
-        const C ih = prm<C>(cd.inv_h[a], cd.f.inv_h[a]);
-        for (int f = 0; f < 6; ++f) rhs[f] += (fe[f] - fw[f]) * ih;
-        gu[0][a] = (C)0.5 * ((R.u - P.u) * ih + (P.u - L.u) * ih);
-        gu[1][a] = (C)0.5 * ((R.v - P.v) * ih + (P.v - L.v) * ih);
-        gu[2][a] = (C)0.5 * ((R.w - P.w) * ih + (P.w - L.w) * ih);
-        if (kl == FK_WALL || kr == FK_WALL) {
+    auto nut_at = [&](const St<C>& s, int c) { return nutf ? to_c<C>(ldg(nutf + c)) : nut_of(s.k, s.om, nu); };
+    int c = ic + sy * jc + sz * k0;
+    St<C> P = load_state<S, C>(in, c);
+    C nutP = nut_at(P, c);
+    uint32_t f = __ldg(cd.nbf0 + c);
+    Face<C> zlo = {};
+    if (cd.active[2] && !(f & 0x1300u)) {   // the first plane's lower face inside the grid
+        const St<C> B = load_state<S, C>(in, c - sz);
+        face_of<2>(cd, B, P, (C)0.5 * (nutP + nut_at(B, c - sz)), zlo);
+    }
+    for (int k = k0; k < k1; ++k) {
+        const int cn = k + 1 < nz ? c + sz : c;
+        const St<C> N = load_state<S, C>(in, cn);
+        const C nutN = nut_at(N, cn);
+        const uint32_t fn = __ldg(cd.nbf0 + cn);
+        const bool fluid = !(f & 0x1000u);
+        C rhs[6] = {(C)0, (C)0, (C)0, (C)0, (C)0, (C)0};
+        C gu[3][3] = {};
+        C omw = (C)0;
+        auto wall = [&](int a, bool is) {
             const C ow = prm<C>(cd.om_wall[a], cd.f.om_wall[a]);
-            omw = ow > omw ? ow : omw;
+            if (is) omw = ow > omw ? ow : omw;
+        };
+        if (cd.active[0]) {
+            Face<C> lo = {}, hi;
+            bool w = false;
+            if (fluid) {
+                if (!(f & 0x3u)) {
+                    const St<C> L = load_state<S, C>(in, c - 1);
+                    face_of<0>(cd, L, P, (C)0.5 * (nutP + nut_at(L, c - 1)), lo);
+                } else {
+                    w = ghost_face<0, -1, S>(cd, in, ic, jc, k, P, nutP, lo);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 6; ++q) hi.fl[q] = __shfl_down_sync(0xffffffffu, lo.fl[q], 1);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) hi.d[q] = __shfl_down_sync(0xffffffffu, lo.d[q], 1);
+            if (fluid && (f & 0xcu)) w |= ghost_face<0, 1, S>(cd, in, ic, jc, k, P, nutP, hi);
+            add_axis<0>(cd, lo, hi, rhs, gu);
+            wall(0, w);
         }
-    }
-    // S^2 = 2 S_ij S_ij
-    C S2 = (C)0;
-    for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) {
-            const C s = (C)0.5 * (gu[a][b] + gu[b][a]);
-            S2 += s * s;
+        if (cd.active[1]) {
+            Face<C> lo = {}, hi;
+            bool w = false;
+            if (fluid) {
+                if (!(f & 0x30u)) {
+                    const St<C> L = load_state<S, C>(in, c - sy);
+                    face_of<1>(cd, L, P, (C)0.5 * (nutP + nut_at(L, c - sy)), lo);
+                } else {
+                    w = ghost_face<1, -1, S>(cd, in, ic, jc, k, P, nutP, lo);
+                }
+            }
+            C(*const mine)[kRows][32] = rows[k & 1];
+#pragma unroll
+            for (int q = 0; q < 6; ++q) mine[q][row][lane] = lo.fl[q];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) mine[6 + q][row][lane] = lo.d[q];
+            __syncthreads();
+            if (row + 1 < nrows) {
+#pragma unroll
+                for (int q = 0; q < 6; ++q) hi.fl[q] = mine[q][row + 1][lane];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) hi.d[q] = mine[6 + q][row + 1][lane];
+            } else if (fluid && !(f & 0xc0u)) {
+                const St<C> R = load_state<S, C>(in, c + sy);
+                face_of<1>(cd, P, R, (C)0.5 * (nutP + nut_at(R, c + sy)), hi);
+            } else {
+                hi = lo;
+            }
+            if (fluid && (f & 0xc0u)) w |= ghost_face<1, 1, S>(cd, in, ic, jc, k, P, nutP, hi);
+            add_axis<1>(cd, lo, hi, rhs, gu);
+            wall(1, w);
         }
-    S2 = (C)2 * S2;
-    C nw[6];
-    exp_update<C>(cd, P, nutP, S2, rhs, dt_of<C>(dt_state, 0), nw);
-    if constexpr (kBlend) {
-        const C a = prm<C>(wb, wbf), b = prm<C>(ws, wsf);
-        for (int f = 0; f < 6; ++f) nw[f] = a * to_c<C>(((const S*)base.f[f])[c]) + b * nw[f];
+        if (cd.active[2]) {
+            Face<C> hi = {};
+            bool w = false;
+            if (fluid && (f & 0x300u)) w = ghost_face<2, -1, S>(cd, in, ic, jc, k, P, nutP, zlo);
+            if (fluid) {
+                if (!(f & 0xc00u)) face_of<2>(cd, P, N, (C)0.5 * (nutP + nutN), hi);
+                else w |= ghost_face<2, 1, S>(cd, in, ic, jc, k, P, nutP, hi);
+            }
+            add_axis<2>(cd, zlo, hi, rhs, gu);
+            wall(2, w);
+            zlo = hi;
+        }
+        if (own) {
+            C nw[6] = {P.u, P.v, P.w, P.T, P.k, P.om};
+            if (fluid) {
+                C S2 = (C)0;   // S^2 = 2 S_ij S_ij
+                for (int a = 0; a < 3; ++a)
+                    for (int b = 0; b < 3; ++b) {
+                        const C s = (C)0.5 * (gu[a][b] + gu[b][a]);
+                        S2 += s * s;
+                    }
+                S2 = (C)2 * S2;
+                exp_update<C>(cd, P, nutP, S2, rhs, dt, nw);
+                if constexpr (kBlend) {
+                    const C a = prm<C>(wb, wbf), b = prm<C>(ws, wsf);
+                    for (int q = 0; q < 6; ++q) nw[q] = a * to_c<C>(((const S*)base.f[q])[c]) + b * nw[q];
+                }
+                if (omw > (C)0) nw[5] = omw;
+            }
+            for (int q = 0; q < 6; ++q) ((S*)out.f[q])[c] = from_c<S, C>(nw[q]);
+        }
+        P = N;
+        nutP = nutN;
+        f = fn;
+        c = cn;
     }
-    if (omw > (C)0) nw[5] = omw;
-    for (int f = 0; f < 6; ++f) o[f][c] = from_c<S, C>(nw[f]);
 }
 
 // ------------------------------------------------------------------ pressure RHS
@@ -1495,15 +1584,36 @@ cudaError_t launch_destruction(int prec, const CaseDev& cd, StatePtrs in, void* 
 
 cudaError_t launch_explicit(int prec, const CaseDev& cd, StatePtrs in, StatePtrs out, const double* dt_state,
                             const void* nut, StatePtrs base, double wb, double ws, cudaStream_t s) {
+    constexpr int kCells = ExplicitK<float, float, false>::kCells;
+    // rows per block: eight, or fewer on a single plane's worth of columns that would leave half the
+    // SMs without a block (FP64 128 x 32 x 1: 26 us with eight rows, 17.5 with two).  Always eight in
+    // a batch, whose merged launch has one block shape.
+    int rows = ExplicitK<float, float, false>::kRows;
+    auto columns = [&](int r) { return (int64_t)((cd.n[0] + kCells - 1) / kCells) * ((cd.n[1] + r - 1) / r); };
+    if (!g_rec)
+        while (rows > 2 && columns(rows) * cd.n[2] < 76) rows /= 2;
+    // planes per block: the longest march (a march loads one plane and forms one layer of faces more
+    // than it owns) of at most 16 that leaves 1000 blocks, counted over a batch's cases.  FP32
+    // 256 x 64 x 64: 33.7 us with 4 (1152 blocks), 36 with 8; 512 x 128 x 128: 199 / 203 / 220 us
+    // with 8 / 16 / 32.
+    int zc = 1;
+    for (int z : {16, 8, 4, 2})
+        if (columns(rows) * ((cd.n[2] + z - 1) / z) * (g_rec ? g_rec->cases : 1) >= 1000) {
+            zc = z;
+            break;
+        }
+    const dim3 grid((unsigned)((cd.n[0] + kCells - 1) / kCells), (unsigned)((cd.n[1] + rows - 1) / rows),
+                    (unsigned)((cd.n[2] + zc - 1) / zc));
+    const dim3 block(32, (unsigned)rows);
     cudaError_t err = cudaSuccess;
     if (base.f[0])
         DISPATCH(prec, err = launch_k(ExplicitK<S, C, true>{cd, in, out, dt_state, (const S*)nut, base, wb, ws,
-                                                            (float)wb, (float)ws},
-                                      grid3(cd), kBlock3, 0, s));
+                                                            (float)wb, (float)ws, zc, 0},
+                                      grid, block, 0, s));
     else
         DISPATCH(prec, err = launch_k(ExplicitK<S, C, false>{cd, in, out, dt_state, (const S*)nut, base, wb, ws,
-                                                             (float)wb, (float)ws},
-                                      grid3(cd), kBlock3, 0, s));
+                                                             (float)wb, (float)ws, zc, 0},
+                                      grid, block, 0, s));
     return err;
 }
 
