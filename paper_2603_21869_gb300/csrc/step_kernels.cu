@@ -155,6 +155,17 @@ template <class C>
 __device__ __forceinline__ C nut_of(C k, C om, C nu) {
     return qdiv(alpha_star_of(re_t(k, om, nu)) * k, omega_safe(om));
 }
+// FP64: the same as one quotient, k (R_k alpha*_0 n + k) / (omega (R_k n + k)) with n = nu omega
+// (alpha*_inf = 1).  An FP64 quotient takes about ten instructions of a pipe with a 64th of the FP32
+// rate, so the FP64 closures below keep numerators and denominators apart and divide once a result:
+// 256 x 64 x 64, us a launch: destruction 502 -> 258, with the right-hand side 451 -> 249,
+// explicit stage 717 -> 567, time-step bound 117 -> 65.  FP32 divides as it goes (__fdividef is two instructions).
+template <>
+__device__ __forceinline__ double nut_of<double>(double k, double om, double nu) {
+    static_assert(kAlphaStarInf == 1.0, "alpha*_inf is a factor of nu_t");
+    const double oms = omega_safe(om), n = nu * oms;
+    return k * (kRk * kAlphaStar0 * n + k) / (oms * (kRk * n + k));
+}
 
 // ------------------------------------------------------------------ init
 __device__ __forceinline__ uint64_t splitmix64_at(uint64_t seed, uint64_t n) {
@@ -185,6 +196,19 @@ __global__ void k_init(CaseDev cd, StatePtrs st, double b0, double b1, double b2
 }
 
 // ------------------------------------------------------------------ dt
+// the warp's largest value of a non-negative lam (no NaN), in every lane; in FP64 as integers, which
+// order alike, the upper words first
+__device__ __forceinline__ float warp_max(float lam) {
+    for (int off = 16; off > 0; off >>= 1) lam = fmaxf(lam, __shfl_xor_sync(0xffffffffu, lam, off));
+    return lam;
+}
+__device__ __forceinline__ double warp_max(double lam) {
+    const unsigned hi = (unsigned)__double2hiint(lam) & 0x7fffffffu;   // -0 is 0
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)__double2loint(lam) : 0u);
+    return __hiloint2double((int)mh, (int)ml);
+}
+
 // rate = sum_active (|u_a| / h_a + 2 Gamma / h_a^2), Gamma = max(nu + nu_t, alpha + nu_t / Pr_t);
 // the block maxima go to dt_state[3] (as ordered bits of a non-negative double)
 template <class S, class C>
@@ -215,7 +239,7 @@ __device__ void RateMaxK<S, C>::run(const BlockAt& at) const {
         lam = l == l ? l : (C)INFINITY;   // NaN -> +inf
     }
     __shared__ double red[kThreads / 32];
-    for (int off = 16; off > 0; off >>= 1) lam = fmax(lam, __shfl_xor_sync(0xffffffffu, lam, off));
+    lam = warp_max(lam);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = (double)lam;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -309,6 +333,39 @@ __device__ __forceinline__ void des_update(const C gu[3][3], C gkw, C k, C om, C
     omnew = qdiv(om, (C)1 + dt * (C)kBeta * fb * om);
 }
 
+// FP64: one reciprocal of nu omega and one quotient for k and for omega each (nut_of); the limits of
+// chi_k, Re_t and chi_omega above keep every product in range
+template <>
+__device__ __forceinline__ void des_update<double>(const double gu[3][3], double gkw, double k, double om, double nu,
+                                                   double dt, double& knew, double& omnew) {
+    const double rn = 1.0 / (nu * omega_safe(om)), r = rn * nu;   // 1 / (nu omega), 1 / omega
+    const double r3 = r * r * r;
+    const double chik = gkw * r3;
+    double fn = 1.0, fd = 1.0;   // f_beta* = fn / fd
+    if (chik > 0.0) {
+        const double c2 = chik * chik;
+        const bool lim = chik > 1e8;
+        fn = lim ? 680.0 : 1.0 + 680.0 * c2;
+        fd = lim ? 400.0 : 1.0 + 400.0 * c2;
+    }
+    const double x = k * rn * (1.0 / kRbeta);
+    const double x2 = x * x, x4 = x2 * x2;
+    const bool turb = x > 1e4;
+    const double bn = turb ? 1.0 : 4.0 / 15.0 + x4, bd = turb ? 1.0 : 1.0 + x4;   // beta* / beta*_inf = bn / bd
+    const double dk = bd * fd;
+    knew = k * dk / (dk + dt * kBetaStarInf * (bn * fn) * om);
+    // four times the trace below: w and the off-diagonal S without their factors 1/2
+    const double w1 = gu[2][1] - gu[1][2], w2 = gu[0][2] - gu[2][0], w3 = gu[1][0] - gu[0][1];
+    const double s01 = gu[0][1] + gu[1][0], s02 = gu[0][2] + gu[2][0], s12 = gu[1][2] + gu[2][1];
+    const double q1 = w1 * w1, q2 = w2 * w2, q3 = w3 * w3;
+    const double tr = w1 * (w2 * s01 + w3 * s02) + w2 * w3 * s12 - (q2 + q3) * gu[0][0] - (q1 + q3) * gu[1][1] -
+                      (q1 + q2) * gu[2][2];
+    const double chiw = fabs(tr * r3) * (0.25 / (kBetaStarInf * kBetaStarInf * kBetaStarInf));
+    const bool far = chiw > 1e30;   // f_beta = wn / wd
+    const double wn = far ? 70.0 : 1.0 + 70.0 * chiw, wd = far ? 80.0 : 1.0 + 80.0 * chiw;
+    omnew = om * wd / (wd + dt * kBeta * wn * om);
+}
+
 template <class S, class C>
 __device__ void DestructionK<S, C>::run(const BlockAt& at) const {
     int i, j, k;
@@ -345,6 +402,16 @@ __device__ void DestructionK<S, C>::cell(int i, int j, int k) const {
             neighbour<S, C>(cd, in, i, j, k, a, +1, P, R);
         }
         const C ih = prm<C>(cd.inv_h[a], cd.f.inv_h[a]);
+        if constexpr (sizeof(C) == 8) {   // the FP64 pipe: two instructions a gradient, div u their trace
+            const C hh = (C)0.5 * ih;
+            gu[0][a] = (R.u - L.u) * hh;
+            gu[1][a] = (R.v - L.v) * hh;
+            gu[2][a] = (R.w - L.w) * hh;
+            gk[a] = (R.k - L.k) * hh;
+            gw[a] = (R.om - L.om) * hh;
+            div += gu[a][a];
+            continue;
+        }
         gu[0][a] = (C)0.5 * ((R.u - P.u) * ih + (P.u - L.u) * ih);
         gu[1][a] = (C)0.5 * ((R.v - P.v) * ih + (P.v - L.v) * ih);
         gu[2][a] = (C)0.5 * ((R.w - P.w) * ih + (P.w - L.w) * ih);
@@ -451,6 +518,17 @@ __device__ __forceinline__ void face_flux(const CaseDev& cd, int a, const St<C>&
     const C gT = prm<C>(cd.alpha, cd.f.alpha) + nut_f * prm<C>(cd.inv_Prt, cd.f.inv_Prt);
     const C gk = nu + nut_f * prm<C>(cd.inv_sigk, cd.f.inv_sigk);
     const C gw = nu + nut_f * prm<C>(cd.inv_sigw, cd.f.inv_sigw);
+    if constexpr (sizeof(C) == 8) {   // Gamma / h once for three momenta: 18 instructions of the pipe, not 24
+        const C mh = gm * ih;
+        fl[0] = mh * (R.u - L.u) - (pos ? L.u : R.u) * uf;
+        fl[1] = mh * (R.v - L.v) - (pos ? L.v : R.v) * uf;
+        fl[2] = mh * (R.w - L.w) - (pos ? L.w : R.w) * uf;
+        fl[3] = gT * ih * (R.T - L.T) - (pos ? L.T : R.T) * uf;
+        fl[4] = gk * ih * (R.k - L.k) - (pos ? L.k : R.k) * uf;
+        fl[5] = gw * ih * (R.om - L.om) - (pos ? L.om : R.om) * uf;
+        fl[a] -= (C)(1.0 / 3.0) * (L.k + R.k);
+        return;
+    }
     fl[0] = -((pos ? L.u : R.u) * uf) + gm * (R.u - L.u) * ih;
     fl[1] = -((pos ? L.v : R.v) * uf) + gm * (R.v - L.v) * ih;
     fl[2] = -((pos ? L.w : R.w) * uf) + gm * (R.w - L.w) * ih;
@@ -471,7 +549,8 @@ __device__ __forceinline__ void face_flux(const CaseDev& cd, int a, const St<C>&
 // the FP32 rate); a thread a cell computed every inner face twice.  One cell a thread -> this, us a
 // launch: FP32 256 x 64 x 64 36.8 -> 33.7, 512 x 128 x 128 266 -> 203, BF16-mixed room
 // 512 x 256 x 128 522 -> 389, eight FP32 channels of 256 x 64 x 64 in a batch 277 -> 208; FP64
-// 256 x 64 x 64 770 -> 718 (at 128 registers; 747 with one block an SM and no spills).
+// 256 x 64 x 64 770 -> 717 (at 128 registers; 747 with one block an SM and no spills), and 567 with
+// fewer quotients (nut_of).
 template <class S, class C, bool kBlend>
 struct ExplicitK {
     static constexpr int kThreads = 256, kRows = 8, kCells = 31;
@@ -499,11 +578,18 @@ template <class C>
 __device__ __forceinline__ void exp_update(const CaseDev& cd, const St<C>& P, C nutP, C S2, C rhs[6], C dt, C o[6]) {
     const C nu = prm<C>(cd.nu, cd.f.nu);
     const C Gk = nutP * S2;
-    const C ret = re_t(P.k, P.om, nu);
-    const C rw = qdiv(ret, (C)kRw);
-    const C alpha = qdiv((C)kAlphaInf, alpha_star_of(ret)) * qdiv((C)kAlpha0 + rw, (C)1 + rw);
     rhs[4] += Gk;
-    rhs[5] += qdiv(alpha * P.om, P.k) * Gk;
+    if constexpr (sizeof(C) == 8) {   // alpha omega / k G_k as one quotient (nut_of)
+        const C n = nu * omega_safe(P.om);
+        const C num = (C)kAlphaInf * P.om * ((C)kRk * n + P.k) * ((C)(kRw * kAlpha0) * n + P.k);
+        const C den = P.k * ((C)(kRk * kAlphaStar0) * n + P.k) * ((C)kRw * n + P.k);
+        rhs[5] += num / den * Gk;
+    } else {
+        const C ret = re_t(P.k, P.om, nu);
+        const C rw = qdiv(ret, (C)kRw);
+        const C alpha = qdiv((C)kAlphaInf, alpha_star_of(ret)) * qdiv((C)kAlpha0 + rw, (C)1 + rw);
+        rhs[5] += qdiv(alpha * P.om, P.k) * Gk;
+    }
     const C dT = P.T - prm<C>(cd.T_ref, cd.f.T_ref);
     rhs[0] += prm<C>(cd.gb[0], cd.f.gb[0]) * dT;
     rhs[1] += prm<C>(cd.gb[1], cd.f.gb[1]) * dT;
@@ -552,7 +638,8 @@ __device__ __forceinline__ void add_axis(const CaseDev& cd, const Face<C>& lo, c
 #pragma unroll
     for (int f = 0; f < 6; ++f) rhs[f] += (hi.fl[f] - lo.fl[f]) * ih;
 #pragma unroll
-    for (int v = 0; v < 3; ++v) gu[v][A] = (C)0.5 * (hi.d[v] * ih + lo.d[v] * ih);
+    for (int v = 0; v < 3; ++v)
+        gu[v][A] = sizeof(C) == 8 ? (hi.d[v] + lo.d[v]) * ((C)0.5 * ih) : (C)0.5 * (hi.d[v] * ih + lo.d[v] * ih);
 }
 
 template <class S, class C, bool kBlend>
