@@ -58,6 +58,7 @@ struct CoarseK {
     C w[2][kMaxChebSweeps];  // smoother 1: the weight of sweep i before (0) and after (1) the coarse correction
     const TI* r_in;
     TI* e_out;
+    double* p;               // the finest level is level 0: its correction is added to p (else null)
     const double* Ainv;
     const SolveState* st;
 };
@@ -709,7 +710,17 @@ struct Body {
             const int own = s.own;
             const C* const v = sm + s.e0 + ((cur & 1u) ? s.flip : 0);
             TI* const out = k.e_out + s.base;
-            if (s.P % 4 == 0)
+            if (k.p) {
+                double* const p = k.p + s.base;   // (pairs where the corrections are not FP64: pp_load)
+                for (int c = tid; c < own; c += T) {
+                    if constexpr (sizeof(C) == 8) {
+                        p[c] += v[c];
+                    } else {
+                        float2* const q = reinterpret_cast<float2*>(p) + c;
+                        *q = pp_plus(*q, v[c]);
+                    }
+                }
+            } else if (s.P % 4 == 0)
                 for (int c = 4 * tid; c < own; c += 4 * T) store4(out + c, load4(v + c));
             else
                 for (int c = tid; c < own; c += T) out[c] = from_c<TI, C>(v[c]);
@@ -806,7 +817,8 @@ cudaError_t coarse_many(const void* tab, const BatchMap& m, unsigned nblk, dim3,
 }
 
 template <class TI>
-CoarseK<TI> functor(const CoarsePlan& pl, const void* r_in, void* e_out, const double* Ainv, const SolveState* st) {
+CoarseK<TI> functor(const CoarsePlan& pl, const void* r_in, void* e_out, double* p, const double* Ainv,
+                    const SolveState* st) {
     using C = typename Acc<TI>::type;
     CoarseK<TI> k;
     memset(&k, 0, sizeof(k));
@@ -845,15 +857,16 @@ CoarseK<TI> functor(const CoarsePlan& pl, const void* r_in, void* e_out, const d
         for (int i = 0; i < kMaxChebSweeps; ++i) k.w[side][i] = (C)pl.w[side][i];
     k.r_in = (const TI*)r_in;
     k.e_out = (TI*)e_out;
+    k.p = p;
     k.Ainv = Ainv;
     k.st = st;
     return k;
 }
 
 template <class TI>
-cudaError_t launch(const CoarsePlan& pl, const void* r_in, void* e_out, const double* Ainv, const SolveState* st,
-                   cudaStream_t s) {
-    const CoarseK<TI> k = functor<TI>(pl, r_in, e_out, Ainv, st);
+cudaError_t launch(const CoarsePlan& pl, const void* r_in, void* e_out, double* p, const double* Ainv,
+                   const SolveState* st, cudaStream_t s) {
+    const CoarseK<TI> k = functor<TI>(pl, r_in, e_out, p, Ainv, st);
     if (record_launch(k, dim3((unsigned)pl.S), dim3(kCtaThreads), pl.smem, &coarse_many<TI>)) return cudaSuccess;
     const void* fn = (const void*)k_coarse<TI>;
     if (!smem_limit_covers(fn, pl.smem)) return cudaErrorInvalidConfiguration;
@@ -937,8 +950,18 @@ static bool plan_from(const std::vector<LevelDev>& levels, const std::vector<uin
 }
 
 bool coarse_plan(const std::vector<LevelDev>& levels, const std::vector<uint32_t>& dir, int inner, int S, bool exact,
-                 CoarsePlan& pl) {
-    for (int lc = 1; lc < (int)levels.size(); ++lc) {
+                 int first, CoarsePlan& pl) {
+    // level 0 itself: where its cells go through the four-cell forms as much as any level, else half of
+    // that in FP64 and a quarter in FP32 and BF16.  Ten steps of six V-cycles, level 0 in the cluster
+    // against in launches: FP64 plane of 4096 cells 3.88 / 4.10 ms, of 8192 4.28 / 4.28, FP64 box of 8192
+    // 5.06 / 5.13; FP32 boxes of 8192 cells 2.50 / 2.75, 32,768 2.84 / 3.13, 65,536 3.19 / 3.29, plane of
+    // 8192 2.73 / 2.93, of 16,384 3.09 / 3.25, of 32,768 3.41 / 3.30
+    if (first == 0) {
+        const LevelDev& v = levels[0];
+        const bool quads = v.active[0] && v.active[1] && v.active[2] && v.n[0] % 4 == 0;
+        if (!quads && v.N > cells_per_block(inner, S) * S / (inner == FVM_FP64 ? 2 : 4)) first = 1;
+    }
+    for (int lc = first; lc < (int)levels.size(); ++lc) {
         if (!plan_from(levels, dir, inner, S, lc, pl)) continue;
         if (exact || S == 1 || pl.lm > 0 || pl.nl == 1) return true;
         return plan_from(levels, dir, inner, 1, lc, pl) || plan_from(levels, dir, inner, S, lc, pl);
@@ -959,9 +982,9 @@ cudaError_t prepare_coarse(int inner, const CoarsePlan& pl) {
     return prepare_kernel(fn, pl.S, pl.smem);
 }
 
-cudaError_t launch_coarse(int inner, const CoarsePlan& pl, const void* r_in, void* e_out, const double* Ainv,
-                          const SolveState* st, cudaStream_t s) {
-    if (inner == FVM_FP64) return launch<double>(pl, r_in, e_out, Ainv, st, s);
-    if (inner == FVM_FP32) return launch<float>(pl, r_in, e_out, Ainv, st, s);
-    return launch<__nv_bfloat16>(pl, r_in, e_out, Ainv, st, s);
+cudaError_t launch_coarse(int inner, const CoarsePlan& pl, const void* r_in, void* e_out, double* p,
+                          const double* Ainv, const SolveState* st, cudaStream_t s) {
+    if (inner == FVM_FP64) return launch<double>(pl, r_in, e_out, p, Ainv, st, s);
+    if (inner == FVM_FP32) return launch<float>(pl, r_in, e_out, p, Ainv, st, s);
+    return launch<__nv_bfloat16>(pl, r_in, e_out, p, Ainv, st, s);
 }

@@ -369,9 +369,10 @@ cudaError_t launch_resid_restrict(int inner, const LevelDev& Lf, const LevelDev&
 cudaError_t launch_prolong_add(int inner, const LevelDev& Lf, const LevelDev& Lc, const void* ec, void* e,
                                const SolveState* st, cudaStream_t s);
 // the cluster's share of the levels: the finest level that a cluster of S blocks takes (S smaller
-// where that leaves nothing to deal out, unless exact), the partition and the layout
+// where that leaves nothing to deal out, unless exact), the partition and the layout; first: the
+// finest level that may be among them
 bool coarse_plan(const std::vector<LevelDev>& levels, const std::vector<uint32_t>& dir, int inner, int S, bool exact,
-                 CoarsePlan& pl);
+                 int first, CoarsePlan& pl);
 int coarse_cluster_for(int cases);   // blocks per cluster when this many cases run theirs at once
 // sets the kernel's limits; an error where the device cannot run such a cluster
 cudaError_t prepare_coarse(int inner, const CoarsePlan& pl);
@@ -391,8 +392,9 @@ cudaError_t launch_prolong_nearest_to_p(int inner, const LevelDev& Lf, const Lev
                                         const SolveState* st, cudaStream_t s);
 cudaError_t launch_jacobi_p(int bprec, const LevelDev& L, double* p, const void* b, double* q, const SolveState* st,
                             cudaStream_t s);
-cudaError_t launch_coarse(int inner, const CoarsePlan& pl, const void* r_in, void* e_out, const double* Ainv,
-                          const SolveState* st, cudaStream_t s);
+// the cluster's levels from r_in, their correction to e_out or (level 0 among them: p not null) added to p
+cudaError_t launch_coarse(int inner, const CoarsePlan& pl, const void* r_in, void* e_out, double* p,
+                          const double* Ainv, const SolveState* st, cudaStream_t s);
 cudaError_t launch_convert(int src_prec, int dst_prec, const void* src, void* dst, int64_t N, cudaStream_t s);
 int resid0_blocks(int nx, int ny, int nz);
 int level0_blocks_max(int nx, int ny, int nz);   // blocks of any level-0 reduction pass, at most

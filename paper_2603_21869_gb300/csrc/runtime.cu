@@ -802,7 +802,7 @@ fvm_status cycle(fvm_case* c, size_t l, int& out_idx) {
         double cells = 0.0;
         for (size_t q = l; q < c->levels.size(); ++q) cells += (double)c->levels[q].dev.N;
         KLAUNCH("coarse_cta", 2 * N * si + nco * nco * 8 + 2 * cells, 1,
-                launch_coarse(c->inner, cp, L.r, L.e[0], c->Ainv, c->sst, s));
+                launch_coarse(c->inner, cp, L.r, L.e[0], l == 0 ? c->p : nullptr, c->Ainv, c->sst, s));
         out_idx = 0;
         return FVM_OK;
     }
@@ -1118,8 +1118,12 @@ int field_slot(int fid) {
 bool plan_coarse_levels(fvm_case* c, int S, bool exact, CoarsePlan& cp) {
     std::vector<LevelDev> lv;
     for (const DevLevel& L : c->levels) lv.push_back(L.dev);
-    if (!coarse_plan(lv, c->level_dir, c->inner, S, exact, cp)) return false;
     const fvm_case_desc& d = c->desc;
+    // level 0 is among them (where it fits) when the whole cycle is one V-cycle whose correction goes
+    // straight to p and whose levels sweep alike; in a batch the cases share level 0's launches
+    const bool whole = !exact && d.mg_variant == 0 && d.krylov == 0 && c->inner_cycles == 1 &&
+                       (d.coarse_sweeps == 0 || (d.coarse_sweeps == d.pre_sweeps && d.coarse_sweeps == d.post_sweeps));
+    if (!coarse_plan(lv, c->level_dir, c->inner, S, exact, whole ? 0 : 1, cp)) return false;
     cp.pre = d.coarse_sweeps > 0 ? d.coarse_sweeps : d.pre_sweeps;   // (levels below the finest)
     cp.post = d.coarse_sweeps > 0 ? d.coarse_sweeps : d.post_sweeps;
     cp.cheb = d.smoother == 1 ? 1 : 0;
