@@ -571,6 +571,12 @@ struct ExplicitK {
     __device__ void run(const BlockAt& at) const;
 };
 
+// alpha omega / k, the ratio of the production terms of omega and k (Eqs. o_gen, a), as one FP64 quotient
+__device__ __forceinline__ double production_ratio(double k, double om, double nu) {
+    const double n = nu * omega_safe(om);
+    return kAlphaInf * om * (kRk * n + k) * (kRw * kAlpha0 * n + k) / (k * (kRk * kAlphaStar0 * n + k) * (kRw * n + k));
+}
+
 // The cell update of the explicit stage from the summed face fluxes rhs (Algorithm 2): the
 // production of k and omega (Eqs. k_gen, o_gen, a) with S2 = 2 S_ij S_ij, Boussinesq buoyancy
 // -g beta_T (T - T_ref), the forward-Euler step dt and the lower bounds of k and omega
@@ -580,10 +586,7 @@ __device__ __forceinline__ void exp_update(const CaseDev& cd, const St<C>& P, C 
     const C Gk = nutP * S2;
     rhs[4] += Gk;
     if constexpr (sizeof(C) == 8) {   // alpha omega / k G_k as one quotient (nut_of)
-        const C n = nu * omega_safe(P.om);
-        const C num = (C)kAlphaInf * P.om * ((C)kRk * n + P.k) * ((C)(kRw * kAlpha0) * n + P.k);
-        const C den = P.k * ((C)(kRk * kAlphaStar0) * n + P.k) * ((C)kRw * n + P.k);
-        rhs[5] += num / den * Gk;
+        rhs[5] += production_ratio(P.k, P.om, nu) * Gk;
     } else {
         const C ret = re_t(P.k, P.om, nu);
         const C rw = qdiv(ret, (C)kRw);
@@ -1110,6 +1113,7 @@ __device__ __forceinline__ double ghost_sign(int f, int kind, int thermal) {
 __device__ __forceinline__ void cell_gradients(const CaseDev& cd, const StatePtrs& in, int i, int j, int k,
                                                const St<double>& P, double (&gu)[3][3], double (&gk)[3],
                                                double (&gw)[3]) {
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
         if (!cd.active[a]) {
             gu[0][a] = gu[1][a] = gu[2][a] = gk[a] = gw[a] = 0.0;
@@ -1118,12 +1122,12 @@ __device__ __forceinline__ void cell_gradients(const CaseDev& cd, const StatePtr
         St<double> L, R;
         neighbour<double, double>(cd, in, i, j, k, a, -1, P, L);
         neighbour<double, double>(cd, in, i, j, k, a, +1, P, R);
-        const double ih = cd.inv_h[a];
-        gu[0][a] = 0.5 * ((R.u - P.u) * ih + (P.u - L.u) * ih);
-        gu[1][a] = 0.5 * ((R.v - P.v) * ih + (P.v - L.v) * ih);
-        gu[2][a] = 0.5 * ((R.w - P.w) * ih + (P.w - L.w) * ih);
-        gk[a] = 0.5 * ((R.k - P.k) * ih + (P.k - L.k) * ih);
-        gw[a] = 0.5 * ((R.om - P.om) * ih + (P.om - L.om) * ih);
+        const double hh = 0.5 * cd.inv_h[a];
+        gu[0][a] = (R.u - L.u) * hh;
+        gu[1][a] = (R.v - L.v) * hh;
+        gu[2][a] = (R.w - L.w) * hh;
+        gk[a] = (R.k - L.k) * hh;
+        gw[a] = (R.om - L.om) * hh;
     }
 }
 
@@ -1133,9 +1137,11 @@ __device__ __forceinline__ void cell_gradients(const CaseDev& cd, const StatePtr
 template <class G>
 __device__ __forceinline__ double gradient_transpose(const CaseDev& cd, int f, int i, int j, int k, int q, G gb) {
     double acc = 0.0;
+#pragma unroll
     for (int m = 0; m < 3; ++m) {
         if (!cd.active[m]) continue;
         const double c2 = 0.5 * cd.inv_h[m];
+#pragma unroll
         for (int side = -1; side <= 1; side += 2) {
             int thermal, nb;
             const int kind = face_kind_of(cd, i, j, k, m, side, thermal, nb);
@@ -1148,7 +1154,9 @@ __device__ __forceinline__ double gradient_transpose(const CaseDev& cd, int f, i
 
 // pass 1 of the destruction adjoint: per cell the partial derivatives of (k', omega') and
 // the cotangents of the 15 gradient components, gbar = [G (3 x 3, row = velocity
-// component), grad k, grad omega] (15 N doubles, component-major)
+// component), grad k, grad omega] (15 N doubles, component-major).  The FP64 pipe bounds both passes:
+// six quotients a cell instead of sixteen and the rotation vector instead of 3 x 3 products took
+// the two from 183 to 111 us at 96 x 48 x 32.
 struct DesAdjAK {
     static constexpr int kThreads = BX * BY * BZ;
     static constexpr bool kNoShared = true;
@@ -1180,85 +1188,71 @@ __device__ void DesAdjAK::run(const BlockAt& at) const {
     double G[3][3], gk[3], gw[3];
     cell_gradients(cd, x, i, j, k, P, G, gk, gw);
     const double nu = cd.nu, kk = P.k, om = P.om;
-    const double oms = om > kEpsOmega ? om : kEpsOmega;
     const double doms = om > kEpsOmega ? 1.0 : 0.0;
+    // (quotients by reciprocals, one a denominator: nut_of)
+    const double dre_dk = 1.0 / (nu * omega_safe(om)), r = dre_dk * nu;   // 1 / (nu omega), 1 / omega
     // k' = k / Dk, Dk = 1 + dt beta* f_beta* omega
-    const double re = kk / (nu * oms), dre_dk = 1.0 / (nu * oms), dre_dom = -re / oms * doms;
-    const double x_ = re / kRbeta, x3 = x_ * x_ * x_, x4 = x3 * x_;
+    const double re = kk * dre_dk, dre_dom = -re * r * doms;
+    const double x_ = re * (1.0 / kRbeta), x3 = x_ * x_ * x_, x4 = x3 * x_;
     double bs, dbs;
     if (x_ > 1e4) {
         bs = kBetaStarInf;
         dbs = 0.0;
     } else {
-        bs = kBetaStarInf * (4.0 / 15.0 + x4) / (1.0 + x4);
-        dbs = kBetaStarInf * (11.0 / 15.0) * 4.0 * x3 / (kRbeta * (1.0 + x4) * (1.0 + x4));   // d beta* / d Re_t
+        const double i4 = 1.0 / (1.0 + x4);
+        bs = kBetaStarInf * (4.0 / 15.0 + x4) * i4;
+        dbs = kBetaStarInf * (11.0 / 15.0) * 4.0 / kRbeta * x3 * (i4 * i4);   // d beta* / d Re_t
     }
     const double dot = gk[0] * gw[0] + gk[1] * gw[1] + gk[2] * gw[2];
-    const double o3 = oms * oms * oms;
-    const double chik = dot / o3;
+    const double r3 = r * r * r;
+    const double chik = dot * r3;
     double fbs = 1.0, dfbs = 0.0;
     if (chik > 0.0 && chik <= 1e8) {
-        const double c2 = chik * chik, d = 1.0 + 400.0 * c2;
-        fbs = (1.0 + 680.0 * c2) / d;
-        dfbs = 560.0 * chik / (d * d);
+        const double c2 = chik * chik, id = 1.0 / (1.0 + 400.0 * c2);
+        fbs = (1.0 + 680.0 * c2) * id;
+        dfbs = 560.0 * chik * (id * id);
     } else if (chik > 1e8) {
         fbs = 680.0 / 400.0;
     }
-    const double Dk = 1.0 + dt * bs * fbs * om;
-    const double ck = -kk / (Dk * Dk) * dt;                    // d k' / d (beta* f_beta* omega)
-    const double dk_dk = 1.0 / Dk + ck * fbs * om * dbs * dre_dk;
-    const double dk_dom = ck * (fbs * om * dbs * dre_dom + bs * om * dfbs * (-3.0 * chik / oms * doms) + bs * fbs);
-    const double dk_dg = ck * bs * om * dfbs / o3;             // times grad omega (for grad k) and grad k
-    // omega' = omega / Dw, Dw = 1 + dt beta f_beta omega, f_beta of chi_w = |T| / (beta*_inf omega_s)^3
-    double S[3][3], O[3][3];
-    for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) {
-            S[a][b] = 0.5 * (G[a][b] + G[b][a]);
-            O[a][b] = 0.5 * (G[a][b] - G[b][a]);
-        }
-    double OO[3][3], SO[3][3], OS[3][3];
-    double T = 0.0;
-    for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) {
-            double s1 = 0.0, s2 = 0.0, s3 = 0.0;
-            for (int e = 0; e < 3; ++e) {
-                s1 += O[a][e] * O[e][b];
-                s2 += S[a][e] * O[e][b];
-                s3 += O[a][e] * S[e][b];
-            }
-            OO[a][b] = s1;
-            SO[a][b] = s2;
-            OS[a][b] = s3;
-        }
-    for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) T += OO[a][b] * S[b][a];
-    const double den = (kBetaStarInf * oms) * (kBetaStarInf * oms) * (kBetaStarInf * oms);
-    const double chiw = fabs(T) / den;
+    const double iDk = 1.0 / (1.0 + dt * bs * fbs * om);
+    const double ck = -kk * (iDk * iDk) * dt;                  // d k' / d (beta* f_beta* omega)
+    const double dk_dk = iDk + ck * fbs * om * dbs * dre_dk;
+    const double dk_dom = ck * (fbs * om * dbs * dre_dom + bs * om * dfbs * (-3.0 * chik * r * doms) + bs * fbs);
+    const double dk_dg = ck * bs * om * dfbs * r3;             // times grad omega (for grad k) and grad k
+    // omega' = omega / Dw, Dw = 1 + dt beta f_beta omega, f_beta of chi_w = |T| / (beta*_inf omega_s)^3,
+    // T = w^T S w - |w|^2 tr S with the rotation vector w (des_update)
+    const double w[3] = {0.5 * (G[2][1] - G[1][2]), 0.5 * (G[0][2] - G[2][0]), 0.5 * (G[1][0] - G[0][1])};
+    const double s01 = 0.5 * (G[0][1] + G[1][0]), s02 = 0.5 * (G[0][2] + G[2][0]), s12 = 0.5 * (G[1][2] + G[2][1]);
+    const double Sw[3] = {G[0][0] * w[0] + s01 * w[1] + s02 * w[2], s01 * w[0] + G[1][1] * w[1] + s12 * w[2],
+                          s02 * w[0] + s12 * w[1] + G[2][2] * w[2]};
+    const double w2 = w[0] * w[0] + w[1] * w[1] + w[2] * w[2], trS = G[0][0] + G[1][1] + G[2][2];
+    const double T = w[0] * Sw[0] + w[1] * Sw[1] + w[2] * Sw[2] - w2 * trS;
+    const double iden = r3 * (1.0 / (kBetaStarInf * kBetaStarInf * kBetaStarInf));
+    const double chiw = fabs(T * iden);
     double fb, dfb;
     if (chiw > 1e30) {
         fb = 70.0 / 80.0;
         dfb = 0.0;
     } else {
-        const double d = 1.0 + 80.0 * chiw;
-        fb = (1.0 + 70.0 * chiw) / d;
-        dfb = -10.0 / (d * d);
+        const double id = 1.0 / (1.0 + 80.0 * chiw);
+        fb = (1.0 + 70.0 * chiw) * id;
+        dfb = -10.0 * (id * id);
     }
     const double sgn = T > 0.0 ? 1.0 : (T < 0.0 ? -1.0 : 0.0);
-    const double Dw = 1.0 + dt * kBeta * fb * om;
-    const double cw = -om / (Dw * Dw) * dt * kBeta;            // d omega' / d (f_beta omega)
-    const double dw_dom = 1.0 / Dw + cw * (fb + om * dfb * (-3.0 * chiw / oms * doms));
-    const double dwg = cw * om * dfb * sgn / den;              // times d T / d G
+    const double iDw = 1.0 / (1.0 + dt * kBeta * fb * om);
+    const double cw = -om * (iDw * iDw) * dt * kBeta;          // d omega' / d (f_beta omega)
+    const double dw_dom = iDw + cw * (fb + om * dfb * (-3.0 * chiw * r * doms));
+    const double dwg = cw * om * dfb * sgn * iden;             // times d T / d G
     kout[c] = kb * dk_dk;
     oout[c] = kb * dk_dom + wb * dw_dom;
-    // d T / d S_ab = (O O)_ba, d T / d O_ab = -(O S + S O)_ab; S, O are the symmetric and
-    // antisymmetric parts of G
-    for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) {
-            const double dS_ab = OO[b][a], dS_ba = OO[a][b];
-            const double dO_ab = -(OS[a][b] + SO[a][b]), dO_ba = -(OS[b][a] + SO[b][a]);
-            const double dT = 0.5 * (dS_ab + dS_ba) + 0.5 * (dO_ab - dO_ba);
-            gbar[(3 * a + b) * N + c] = wb * dwg * dT;
-        }
+    // d T / d G = w w^T - |w|^2 I, from S, and the rotation of v = d T / d w / 2 = S w - tr(S) w, from w
+    // (w_0 = (G_21 - G_12) / 2 and so on round)
+    const double g = wb * dwg;
+    const double v[3] = {Sw[0] - trS * w[0], Sw[1] - trS * w[1], Sw[2] - trS * w[2]};
+    const double p01 = w[0] * w[1], p02 = w[0] * w[2], p12 = w[1] * w[2];
+    const double dT[9] = {w[0] * w[0] - w2, p01 - v[2], p02 + v[1], p01 + v[2], w[1] * w[1] - w2, p12 - v[0],
+                          p02 - v[1], p12 + v[0], w[2] * w[2] - w2};
+    for (int m = 0; m < 9; ++m) gbar[m * N + c] = g * dT[m];
     for (int m = 0; m < 3; ++m) {
         gbar[(9 + m) * N + c] = kb * dk_dg * gw[m];
         gbar[(12 + m) * N + c] = kb * dk_dg * gk[m];
@@ -1289,7 +1283,8 @@ __device__ void DesAdjBK::run(const BlockAt& at) const {
     const bool fluid = cd.tag[c] == 0;
     double acc[5] = {ubar_in[c], ubar_in[N + c], ubar_in[2 * N + c], kout[c], oout[c]};
     if (fluid) {
-        const int field_of[5] = {0, 1, 2, 4, 5};
+        constexpr int field_of[5] = {0, 1, 2, 4, 5};
+#pragma unroll
         for (int v = 0; v < 5; ++v) {
             const double* g = gbar + (size_t)(v < 3 ? 3 * v : (v == 3 ? 9 : 12)) * N;
             acc[v] += gradient_transpose(cd, field_of[v], i, j, k, c,
@@ -1363,9 +1358,7 @@ __device__ void ExpAdjAK::run(const BlockAt& at) const {
     s2[c] = S2;
     const double nu = cd.nu;
     const double nut = nut_of<double>(P.k, P.om, nu);
-    const double ret = re_t<double>(P.k, P.om, nu), rw = ret / kRw;
-    const double alpha = (kAlphaInf / alpha_star_of<double>(ret)) * ((kAlpha0 + rw) / (1.0 + rw));
-    const double q = alpha * P.om / P.k;                       // G_omega = q G_k
+    const double q = production_ratio(P.k, P.om, nu);          // G_omega = q G_k
     const double rk = live_k ? dt * ybar[4 * N + c] : 0.0, ro = live_o ? dt * ybar[5 * N + c] : 0.0;
     const double S2bar = (rk + ro * q) * nut;
     for (int a = 0; a < 3; ++a)
@@ -1376,10 +1369,13 @@ __device__ void ExpAdjAK::run(const BlockAt& at) const {
 // (upwind convection, central diffusion with the face eddy viscosity, the -(2/3) k
 // face term of the normal momentum) transposed onto the cell, the production and
 // buoyancy sources, the eddy viscosity's dependence on k and omega, and the transposed
-// velocity gradient of the production term
+// velocity gradient of the production term.  FP64-pipe bound: four diffusivities a face scaled once,
+// the other side's derivative only where a ghost is built from the cell, one reciprocal a denominator, the
+// axes unrolled (no indexed local arrays): both passes 351 -> 218 us at 96 x 48 x 32.
 struct ExpAdjBK {
     static constexpr int kThreads = BX * BY * BZ;
     static constexpr bool kNoShared = true;
+    static constexpr int kMinBlocks = 2;   // at most 128 registers
     __device__ bool live() const { return true; }
     CaseDev cd;
     StatePtrs x;
@@ -1401,8 +1397,6 @@ __device__ void ExpAdjBK::run(const BlockAt& at) const {
         return;
     }
     const double nu = cd.nu;
-    const double gam[6] = {nu, nu, nu, cd.alpha, nu, nu};
-    const double isig[6] = {1.0, 1.0, 1.0, cd.inv_Prt, cd.inv_sigk, cd.inv_sigw};
     const St<double> P = load_state<double, double>(x, c);
     double rb[6], acc[6];
     // the identity part of phi + dt rhs where the update passes a derivative: there rbar =
@@ -1413,45 +1407,50 @@ __device__ void ExpAdjBK::run(const BlockAt& at) const {
     }
     const double nutP = nut_of<double>(P.k, P.om, nu);
     double nutbar = 0.0;
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
         if (!cd.active[a]) continue;
-        const double ih = cd.inv_h[a];
+        const double ih = cd.inv_h[a], ih2 = ih * ih;
+#pragma unroll
         for (int side = -1; side <= 1; side += 2) {
             int thermal, nb;
             const int kind = face_kind_of(cd, i, j, k, a, side, thermal, nb);
             St<double> Q;   // the state across the face (neighbour or ghost)
             neighbour<double, double>(cd, x, i, j, k, a, side, P, Q);
             const bool interior = kind == FK_INTERIOR;
-            // face cotangents F_bar_f = (rbar(L cell) - rbar(R cell)) / h
+            // face cotangents F_bar_f = (rbar(L cell) - rbar(R cell)) / h; here Fb = h F_bar, with the
+            // coefficients and sums scaled by 1 / h instead (four diffusivities, not six)
             double Fb[6];
             for (int f = 0; f < 6; ++f) {
                 const double rq = interior ? rbar[f * N + nb] : 0.0;
-                Fb[f] = side > 0 ? (rb[f] - rq) * ih : (rq - rb[f]) * ih;
+                Fb[f] = side > 0 ? rb[f] - rq : rq - rb[f];
             }
             const St<double>& L = side > 0 ? P : Q;
             const St<double>& R = side > 0 ? Q : P;
-            const double uf = 0.5 * (vcomp(L, a) + vcomp(R, a));
+            const double uf = 0.5 * (vcomp(L, a) + vcomp(R, a)), uih = uf * ih;
             const bool upL = uf >= 0.0;
             const double nutf = kind == FK_WALL ? 0.0
                                 : (interior ? 0.5 * (nutP + nut_of<double>(Q.k, Q.om, nu)) : nutP);
-            const double phL[6] = {L.u, L.v, L.w, L.T, L.k, L.om}, phR[6] = {R.u, R.v, R.w, R.T, R.k, R.om};
-            double ufb = 0.0, nfb = 0.0;
-            for (int f = 0; f < 6; ++f) {
-                const double G_ = gam[f] + nutf * isig[f];
-                const double dL = Fb[f] * ((upL ? -uf : 0.0) - G_ * ih);
-                const double dR = Fb[f] * ((upL ? 0.0 : -uf) + G_ * ih);
-                // this cell's own side, and (across a ghost face) the ghost built from it
-                double d = side > 0 ? dL : dR;
-                if (!interior) d += ghost_sign(f, kind, thermal) * (side > 0 ? dR : dL);
-                acc[f] += d;
-                ufb += -(upL ? phL[f] : phR[f]) * Fb[f];
-                nfb += (phR[f] - phL[f]) * ih * isig[f] * Fb[f];
-            }
+            const double th = nutf * ih2, nh = nu * ih2;
+            const double gu = nh + th, gT = cd.alpha * ih2 + th * cd.inv_Prt, gk = nh + th * cd.inv_sigk,
+                         gw = nh + th * cd.inv_sigw;
+            // d flux / d phi_L and d phi_R (over h), of this cell's side and of the other one
+            const bool own_up = (side > 0) == upL;
+            const double cu = own_up ? -uih : 0.0, co = own_up ? 0.0 : -uih, sg = side > 0 ? -1.0 : 1.0;
+            const double G[6] = {gu, gu, gu, gT, gk, gw};
+            for (int f = 0; f < 6; ++f) acc[f] += Fb[f] * (cu + sg * G[f]);
+            if (!interior)   // the ghost built from this cell
+                for (int f = 0; f < 6; ++f) acc[f] += Fb[f] * (co - sg * G[f]) * ghost_sign(f, kind, thermal);
+            const double ufb = (upL ? L.u : R.u) * Fb[0] + (upL ? L.v : R.v) * Fb[1] + (upL ? L.w : R.w) * Fb[2] +
+                               (upL ? L.T : R.T) * Fb[3] + (upL ? L.k : R.k) * Fb[4] + (upL ? L.om : R.om) * Fb[5];
+            const double nfb = ih2 * ((R.u - L.u) * Fb[0] + (R.v - L.v) * Fb[1] + (R.w - L.w) * Fb[2] +
+                                      (R.T - L.T) * (Fb[3] * cd.inv_Prt) + (R.k - L.k) * (Fb[4] * cd.inv_sigk) +
+                                      (R.om - L.om) * (Fb[5] * cd.inv_sigw));
             // face velocity (U_L + U_R) / 2 and the -(k_L + k_R) / 3 of the normal momentum
             const double sa = interior ? 0.0 : ghost_sign(a, kind, thermal);
-            acc[a] += 0.5 * ufb * (1.0 + sa);
+            acc[a] -= 0.5 * ih * ufb * (1.0 + sa);
             const double sk = interior ? 0.0 : ghost_sign(4, kind, thermal);
-            acc[4] += -Fb[a] / 3.0 * (1.0 + sk);
+            acc[4] -= ih * (1.0 / 3.0) * Fb[a] * (1.0 + sk);
             // face eddy viscosity: the mean of the two cells inside, this cell's own on
             // inlet, outlet and empty faces, none on walls
             if (interior) nutbar += 0.5 * nfb;
@@ -1461,21 +1460,23 @@ __device__ void ExpAdjBK::run(const BlockAt& at) const {
     // sources: G_k = nu_t S^2, G_omega = q G_k, buoyancy -g_i beta_T (T - T_ref)
     const double S2 = s2[c];
     const double kk = P.k, om = P.om;
-    const double oms = om > kEpsOmega ? om : kEpsOmega, doms = om > kEpsOmega ? 1.0 : 0.0;
-    const double re = kk / (nu * oms), dre_dk = 1.0 / (nu * oms), dre_dom = -re / oms * doms;
-    const double r = re / kRk;
-    const double ast = kAlphaStarInf * (kAlphaStar0 + r) / (1.0 + r);
-    const double dast = kAlphaStarInf * (1.0 - kAlphaStar0) / (kRk * (1.0 + r) * (1.0 + r));
-    const double nut = ast * kk / oms;
-    const double dnut_dk = ast / oms + kk / oms * dast * dre_dk;
-    const double dnut_dom = -ast * kk / (oms * oms) * doms + kk / oms * dast * dre_dom;
-    const double rw = re / kRw;
-    const double A = (kAlpha0 + rw) / (1.0 + rw), dA = (1.0 - kAlpha0) / (kRw * (1.0 + rw) * (1.0 + rw));
-    const double ac = kAlphaInf * A / ast, dac = kAlphaInf * (dA / ast - A * dast / (ast * ast));
+    const double doms = om > kEpsOmega ? 1.0 : 0.0;
+    const double dre_dk = 1.0 / (nu * omega_safe(om)), io = dre_dk * nu;   // 1 / (nu omega), 1 / omega
+    const double re = kk * dre_dk, dre_dom = -re * io * doms;
+    const double r = re * (1.0 / kRk), i1 = 1.0 / (1.0 + r);
+    const double ast = kAlphaStarInf * (kAlphaStar0 + r) * i1;
+    const double dast = kAlphaStarInf * (1.0 - kAlphaStar0) / kRk * (i1 * i1);
+    const double ko = kk * io, nut = ast * ko;
+    const double dnut_dk = ast * io + ko * dast * dre_dk;
+    const double dnut_dom = ko * (dast * dre_dom - ast * io * doms);
+    const double rw = re * (1.0 / kRw), iw = 1.0 / (1.0 + rw);
+    const double A = (kAlpha0 + rw) * iw, dA = (1.0 - kAlpha0) / kRw * (iw * iw);
+    const double ia = 1.0 / ast;
+    const double ac = kAlphaInf * A * ia, dac = ia * (kAlphaInf * dA - ac * dast);
     const double Gk = nut * S2;
-    const double q = ac * om / kk;
-    const double dq_dk = dac * dre_dk * om / kk - ac * om / (kk * kk);
-    const double dq_dom = dac * dre_dom * om / kk + ac / kk;
+    const double ik = 1.0 / kk, q = ac * om * ik;
+    const double dq_dk = om * ik * (dac * dre_dk - ac * ik);
+    const double dq_dom = ik * (dac * dre_dom * om + ac);
     const double rk = rb[4], ro = rb[5];
     acc[4] += ro * Gk * dq_dk;
     acc[5] += ro * Gk * dq_dom;
