@@ -117,7 +117,7 @@ typedef struct {
     int32_t inner_cycles;            /* V-cycles per FP64 outer residual (0: 1 for FP64, 2 otherwise);
                                         the stopping test runs after each group */
     int32_t sweep_planes;            /* z planes per block of the four-cell level kernels, 1..64
-                                        (0: the built-in rule, about eight blocks per SM) */
+                                        (0: the built-in rule by the level's blocks) */
     int32_t mg_variant;              /* 0: V(pre, post) cycles; 1: the paper's scheme (Algorithm 1:
                                         residual restricted straight down, one unweighted Jacobi per
                                         coarse level, nearest upsampling, a final Jacobi on p) */
