@@ -1,4 +1,5 @@
-// The multigrid levels below the grid-wide ones, in one thread-block cluster per V-cycle.
+// The multigrid levels below the grid-wide ones (on a small grid with plain V-cycles, all of them), in
+// one thread-block cluster per V-cycle.
 //
 // A level of a few thousand to some ten thousand cells keeps no GPU busy: run as one launch per
 // sweep or transfer, each launch is a chain of latencies (parameters, face codes, neighbour loads,
