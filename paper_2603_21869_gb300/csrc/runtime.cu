@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "fvm_internal.cuh"
+#include "host_buffer.h"
 
 namespace {
 
@@ -2040,8 +2041,10 @@ fvm_status fvm_read_poisson_rhs(fvm_case* c, double* host_b, size_t n) {
     return FVM_OK;
 }
 
-// the device's address of a pinned (page-locked, mapped) host buffer of n doubles, or null
+// the device's address of a pinned (page-locked, mapped) host buffer of n doubles that a kernel can
+// store into, or null
 static double* pinned_device_pointer(double* host, size_t n) {
+    if (!doubles_aligned((uintptr_t)host)) return nullptr;
     double* dev[2];
     for (int end = 0; end < 2; ++end) {   // both ends: a buffer may reach past what was registered
         double* const at = end ? host + n - 1 : host;
