@@ -3,6 +3,8 @@
 // coarsest-level inverse, device memory, and the order of kernels in one
 // time step (Section 2.6: dt/2 destruction, explicit stage, dt/2
 // destruction, pressure solve, projection).
+#include <cuda.h>
+
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -2041,22 +2043,40 @@ fvm_status fvm_read_poisson_rhs(fvm_case* c, double* host_b, size_t n) {
     return FVM_OK;
 }
 
-// the device's address of a pinned (page-locked, mapped) host buffer of n doubles that a kernel can
-// store into, or null
+// the driver's query of a pointer's allocation (the runtime has none for host memory), or null
+static CUresult (*pointer_attribute())(void*, CUpointer_attribute, CUdeviceptr) {
+    static const auto fn = []() {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return (CUresult(*)(void*, CUpointer_attribute, CUdeviceptr))f;
+    }();
+    return fn;
+}
+
+// the device's address of a host buffer of n doubles in one pinned (page-locked, mapped) allocation
+// that a kernel can store into, or null
 static double* pinned_device_pointer(double* host, size_t n) {
     if (!doubles_aligned((uintptr_t)host)) return nullptr;
-    double* dev[2];
-    for (int end = 0; end < 2; ++end) {   // both ends: a buffer may reach past what was registered
-        double* const at = end ? host + n - 1 : host;
-        cudaPointerAttributes pa;
-        if (cudaPointerGetAttributes(&pa, at) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        if (pa.type != cudaMemoryTypeHost || !pa.devicePointer) return nullptr;
-        dev[end] = (double*)pa.devicePointer;
+    cudaPointerAttributes pa;
+    if (cudaPointerGetAttributes(&pa, host) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
     }
-    return dev[1] - dev[0] == (ptrdiff_t)n - 1 ? dev[0] : nullptr;
+    if (pa.type != cudaMemoryTypeHost || !pa.devicePointer) return nullptr;
+    const auto query = pointer_attribute();
+    const CUdeviceptr at = (CUdeviceptr)(uintptr_t)pa.devicePointer;
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    if (!query || query(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, at) != CUDA_SUCCESS ||
+        query(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, at) != CUDA_SUCCESS ||
+        !allocation_holds((uintptr_t)start, size, (uintptr_t)at, n * sizeof(double)))
+        return nullptr;
+    return (double*)pa.devicePointer;
 }
 
 fvm_status fvm_lambda2(fvm_case* c, double* host_out, size_t n) {
