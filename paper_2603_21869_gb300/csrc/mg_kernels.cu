@@ -22,6 +22,7 @@
 // cycled by one cluster of blocks (coarse_kernels.cu).  The level-0 residual
 // kernel finishes the norm in its last block and decides on the device
 // whether another cycle runs, so the whole solve can live in a CUDA graph.
+#include "fp_convert.h"
 #include "fvm_internal.cuh"
 
 namespace {
@@ -532,6 +533,17 @@ template <> __device__ __forceinline__ void codes_w<8>(const uint16_t* f, int c,
     const uint4 v = __ldg(reinterpret_cast<const uint4*>(f + c));
     o[0] = v.x & 0xffffu; o[1] = v.x >> 16; o[2] = v.y & 0xffffu; o[3] = v.y >> 16;
     o[4] = v.z & 0xffffu; o[5] = v.z >> 16; o[6] = v.w & 0xffffu; o[7] = v.w >> 16;
+}
+
+// two values side by side (aligned to the pair)
+__device__ __forceinline__ void store2(double* p, int c, const double (&v)[2]) {
+    *reinterpret_cast<double2*>(p + c) = make_double2(v[0], v[1]);
+}
+__device__ __forceinline__ void store2(float* p, int c, const float (&v)[2]) {
+    *reinterpret_cast<float2*>(p + c) = make_float2(v[0], v[1]);
+}
+__device__ __forceinline__ void store2(__nv_bfloat16* p, int c, const __nv_bfloat16 (&v)[2]) {
+    *reinterpret_cast<__nv_bfloat162*>(p + c) = __halves2bfloat162(v[0], v[1]);
 }
 
 template <> __device__ __forceinline__ void codes_w<1>(const uint16_t* f, int c, uint32_t (&o)[1]) {
@@ -1159,17 +1171,22 @@ __device__ int Resid0V4K<TI, F>::run(const BlockAt& at) const {
     return resid0_sums<kThreads>((double)r2, (double)b2, partials, st, at);
 }
 
-// r = b - A p, r^2 and b^2 and the first pre-sweep of an FP64 level: two x cells per thread and a z
-// march (the sweep's layout); a thread's squares are summed in registers, one warp reduction a block
-// (the one-cell form's per-cell reduction was 10 of its 24 FP64 operations a cell).
-struct Resid0D2K {
+// r = b - A p, r^2 and b^2 and the first pre-sweep in FP64: two x cells per thread and a z march (the
+// sweep's layout); a thread's squares are summed in registers, one warp reduction a block (the
+// one-cell form's per-cell reduction was 10 of its 24 FP64 operations a cell).  FP64 levels, and the
+// FP32 and BF16 cases under 2^20 cells stepped alone: there p's double-float pairs are summed to FP64
+// and r is rounded once, as in Resid0K (430,080 cells, us a launch: one cell per thread 47, this with
+// conversion instructions 44, with fp_convert.h 32; the double-float form of the large levels 20, with
+// errors of the size of p's last bits).
+template <class TB, class TI>
+struct Resid0DK {
     static constexpr int kThreads = TX * TY;
-    static constexpr int kMinBlocks = 4;
+    static constexpr int kMinBlocks = sizeof(TB) == 8 ? 4 : 3;   // at most 64 registers, 80 with pairs
     LevelDev L;
     const double* p;
-    const double* b;
-    double* r;
-    double* e;
+    const TB* b;
+    TI* r;
+    TI* e;
     double* partials;
     SolveState* st;
     int zc;    // planes per block
@@ -1178,8 +1195,11 @@ struct Resid0D2K {
     __device__ int run(const BlockAt& at) const;
 };
 
-__device__ int Resid0D2K::run(const BlockAt& at) const {
-    using R = RawW<double, 2>;
+template <class TB, class TI>
+__device__ int Resid0DK<TB, TI>::run(const BlockAt& at) const {
+    using C = typename Acc<TI>::type;
+    using R = RawW<double, 2>;   // (a pair has a value's size)
+    using RB = RawW<TB, 2>;
     const int nx = L.n[0], ny = L.n[1], nz = L.n[2];
     const int LR = 1 << lrl, lane = threadIdx.x & (LR - 1), sub = threadIdx.x >> lrl;
     const int i2 = at.b.x * (2 * LR) + lane * 2, j = ((at.b.y * TY + threadIdx.y) << (5 - lrl)) + sub;
@@ -1189,28 +1209,76 @@ __device__ int Resid0D2K::run(const BlockAt& at) const {
     const int ic = min(i2, nx - 2), jc = min(j, ny - 1);
     const int own = ic + sy * jc, om = ic + sy * max(jc - 1, 0), op = ic + sy * min(jc + 1, ny - 1);
     const int xl = max(ic - 1, 0) + sy * jc, xr = min(ic + 2, nx - 1) + sy * jc;
-    const double ihx = L.ih2a[0], ihy = L.ih2a[1], ihz = L.ih2a[2], dg = L.diag, wiD = L.wJ * L.inv_D;
-    double2 em = R::load(p, max(k0 - 1, 0) * sz + own), ec = R::load(p, k0 * sz + own);
+    const double ihx = L.ih2a[0], ihy = L.ih2a[1], ihz = L.ih2a[2], dg = L.diag;
+    // values of p as loaded, in FP64: the values themselves, or the sums of their pairs
+    auto values = [](const auto& raw, auto& v) {
+        constexpr int n = sizeof(v) / sizeof(double);
+        if constexpr (sizeof(TB) == 8) {
+#pragma unroll
+            for (int q = 0; q < n; ++q) v[q] = raw[q];
+        } else {
+            float x[2 * n];
+            double y[2 * n];
+#pragma unroll
+            for (int q = 0; q < n; ++q) {
+                x[2 * q] = __int_as_float(__double2loint(raw[q]));
+                x[2 * q + 1] = __int_as_float(__double2hiint(raw[q]));
+            }
+            widened(x, y);
+#pragma unroll
+            for (int q = 0; q < n; ++q) v[q] = y[2 * q] + y[2 * q + 1];
+        }
+    };
+    double em[2], ec[2];
+    {
+        const double2 a = R::load(p, max(k0 - 1, 0) * sz + own), c = R::load(p, k0 * sz + own);
+        const double raw[4] = {a.x, a.y, c.x, c.y};
+        double v[4];
+        values(raw, v);
+        em[0] = v[0]; em[1] = v[1];
+        ec[0] = v[2]; ec[1] = v[3];
+    }
     double r2 = 0.0, b2 = 0.0;
     for (int k = k0; k < k1; ++k) {
         const int base = k * sz;
-        const double2 ep = R::load(p, min(k + 1, nz - 1) * sz + own);
-        const double2 ym = R::load(p, base + om), yp = R::load(p, base + op), bv = R::load(b, base + own);
-        const double left = __ldg(p + base + xl), right = __ldg(p + base + xr);
+        const double2 e = R::load(p, min(k + 1, nz - 1) * sz + own), m = R::load(p, base + om), q = R::load(p, base + op);
+        const typename RB::T bv = RB::load(b, base + own);
+        const double raw[8] = {e.x, e.y, m.x, m.y, q.x, q.y, __ldg(p + base + xl), __ldg(p + base + xr)};
+        double v[8];   // k + 1; j - 1; j + 1; left, right
+        values(raw, v);
+        const TB bt[2] = {RB::get(bv, 0), RB::get(bv, 1)};
+        double bd[2];
+        widened(bt, bd);
         uint32_t fs[2];
         codes_w<2>(L.nbf, base + own, fs);
-        const double a = resid64(fs[0], bv.x, ec.x, left, ec.y, ym.x, yp.x, em.x, ep.x, ihx, ihy, ihz, dg);
-        const double c = resid64(fs[1], bv.y, ec.y, ec.x, right, ym.y, yp.y, em.y, ep.y, ihx, ihy, ihz, dg);
-        const double ra = is_solid(fs[0]) ? 0.0 : a, rc = is_solid(fs[1]) ? 0.0 : c;
+        const double rd[2] = {resid64(fs[0], bd[0], ec[0], v[6], ec[1], v[2], v[4], em[0], v[0], ihx, ihy, ihz, dg),
+                              resid64(fs[1], bd[1], ec[1], ec[0], v[7], v[3], v[5], em[1], v[1], ihx, ihy, ihz, dg)};
+        C rv[2];
+        narrowed(rd, rv);   // (BF16: by way of FP32, as from_c does)
         if (in) {
-            *reinterpret_cast<double2*>(r + base + own) = make_double2(ra, rc);
-            *reinterpret_cast<double2*>(e + base + own) = make_double2(wiD * ra, wiD * rc);
-            r2 = fma(ra, ra, fma(rc, rc, r2));
-            const double ba = is_solid(fs[0]) ? 0.0 : bv.x, bc = is_solid(fs[1]) ? 0.0 : bv.y;
-            b2 = fma(ba, ba, fma(bc, bc, b2));
+            const TI rs[2] = {from_c<TI, C>(is_solid(fs[0]) ? (C)0 : rv[0]), from_c<TI, C>(is_solid(fs[1]) ? (C)0 : rv[1])};
+            const C va = to_c<C>(rs[0]), vc = to_c<C>(rs[1]);
+            const C ba = is_solid(fs[0]) ? (C)0 : (C)bt[0], bc = is_solid(fs[1]) ? (C)0 : (C)bt[1];
+            const C w = LP<C>::wJ(L), iD = LP<C>::iD(L);
+            store2(r, base + own, rs);
+            if constexpr (sizeof(TI) == 8) {
+                const double wiD = w * iD;
+                const TI es[2] = {wiD * va, wiD * vc};
+                store2(this->e, base + own, es);
+                r2 = fma(va, va, fma(vc, vc, r2));
+                b2 = fma(ba, ba, fma(bc, bc, b2));
+            } else {   // (squares in FP32 as in Resid0K, the sums in FP64)
+                const TI es[2] = {from_c<TI, C>(w * va * iD), from_c<TI, C>(w * vc * iD)};
+                store2(this->e, base + own, es);
+                const float sq[2] = {fmaf(va, va, vc * vc), fmaf(ba, ba, bc * bc)};
+                double sd[2];
+                widened(sq, sd);
+                r2 += sd[0];
+                b2 += sd[1];
+            }
         }
-        em = ec;
-        ec = ep;
+        em[0] = ec[0]; em[1] = ec[1];
+        ec[0] = v[0]; ec[1] = v[1];
     }
     return resid0_sums<kThreads>(r2, b2, partials, st, at);
 }
@@ -1964,9 +2032,8 @@ cudaError_t launch_resid0(int inner, int bprec, const LevelDev& L, const double*
     cudaError_t err = cudaSuccess;
     DISPATCH_I(inner, {
         if constexpr (sizeof(TI) < 8) {
-            // four cells per thread in float-float, whatever the size (430,080 cells: 47 us a launch in
-            // the one-cell form, which works in FP64)
-            if (bprec == FVM_FP32 && L.n[0] % 4 == 0) {
+            // four cells per thread in float-float on large levels and in batches
+            if (bprec == FVM_FP32 && L.n[0] % 4 == 0 && (L.N >= (1 << 20) || g_rec)) {
                 const int lrl = v4_lrl(L.n[0]);
                 int zc = 0;
                 const dim3 grid = v4_grid(L, lrl, zc);
@@ -1978,14 +2045,15 @@ cudaError_t launch_resid0(int inner, int bprec, const LevelDev& L, const double*
                                  dim3(TX, TY), cond, use_cond, s);
             }
         }
-        if constexpr (sizeof(TI) == 8) {
-            if (bprec == FVM_FP64 && L.n[0] % 2 == 0) {
-                const int lrl = vw_lrl(L.n[0], 2);
-                int zc = 0;
-                const dim3 grid = vw_grid(L, 2, lrl, zc);
-                return launch_r0(Resid0D2K{L, p, (const double*)b, (double*)r, (double*)e, partials, st, zc, lrl}, grid,
-                                 dim3(TX, TY), cond, use_cond, s);
-            }
+        // two cells per thread in FP64 on FP64 levels, and on the smaller ones of a reduced-precision
+        // case alone (Resid0DK)
+        using TB = std::conditional_t<sizeof(TI) == 8, double, float>;
+        if (bprec == (sizeof(TI) == 8 ? FVM_FP64 : FVM_FP32) && L.n[0] % (sizeof(TI) == 8 ? 2 : 4) == 0) {
+            const int lrl = vw_lrl(L.n[0], 2);
+            int zc = 0;
+            const dim3 grid = vw_grid(L, 2, lrl, zc);
+            return launch_r0(Resid0DK<TB, TI>{L, p, (const TB*)b, (TI*)r, (TI*)e, partials, st, zc, lrl}, grid,
+                             dim3(TX, TY), cond, use_cond, s);
         }
         if (bprec == FVM_FP64)
             err = launch_r0(Resid0K<double, TI>{L, p, (const double*)b, (TI*)r, (TI*)e, partials, st}, grid3(L),
