@@ -1285,12 +1285,12 @@ __device__ int Resid0DK<TB, TI>::run(const BlockAt& at) const {
 
 // The flexible-CG inner products with W x cells per thread and a z march
 // (the sweep's layout and neighbour scheme): products, the thread's and the
-// warp's sums in FP32, block and grid sums in FP64.  Needs nx % W = 0.
+// warp's sums in T, block and grid sums in FP64.  Needs nx % W = 0.
 // (TR: storage of r; TZ: storage of z and the kept direction, FP32 on BF16 levels)
-template <class TR, class TZ, int W, bool F>   // F: by the group flags
+template <class TR, class TZ, int W, bool F, class T>   // F: by the group flags
 struct FcgDotVK {
     static constexpr int kThreads = TX * TY;
-    static constexpr int kMinBlocks = 4;       // at most 64 registers
+    static constexpr int kMinBlocks = sizeof(T) > sizeof(TZ) ? 3 : 4;   // at most 64 registers (FP64 sums of FP32 fields: 80)
     static constexpr int kMinBlocksMany = 3;   // the batched form: at most 80 registers
     LevelDev L;
     const TZ* z;
@@ -1304,8 +1304,8 @@ struct FcgDotVK {
     __device__ void run(const BlockAt& at) const;
 };
 
-template <class TR, class TZ, int W, bool F>
-__device__ void FcgDotVK<TR, TZ, W, F>::run(const BlockAt& at) const {
+template <class TR, class TZ, int W, bool F, class T>
+__device__ void FcgDotVK<TR, TZ, W, F, T>::run(const BlockAt& at) const {
     using C = typename Acc<TZ>::type;
     using R = RawW<TZ, W>;
     using RR = RawW<TR, W>;
@@ -1327,7 +1327,7 @@ __device__ void FcgDotVK<TR, TZ, W, F>::run(const BlockAt& at) const {
     typename R::T em = R::load(zz, max(k0 - 1, 0) * sz + own);
     typename R::T ec = R::load(zz, k0 * sz + own);
     typename R::T ep = R::load(zz, min(k0 + 1, nz - 1) * sz + own);
-    C a0 = (C)0, a1 = (C)0, a2 = (C)0, a3 = (C)0;
+    T a0 = (T)0, a1 = (T)0, a2 = (T)0, a3 = (T)0;
     for (int k = k0; k < k1; ++k) {
         const int base = k * sz;
         const typename R::T ym = R::load(zz, base + om);
@@ -1372,9 +1372,11 @@ __device__ void FcgDotVK<TR, TZ, W, F>::run(const BlockAt& at) const {
             gf.codes = (any & 0x3000u) != 0u;
         }
         if (in) {
+            C zs[W], As[W], ds[W], rs[W];   // (sums in a wider type: the plane's factors, converted together)
 #pragma unroll
             for (int t = 0; t < W; ++t) {
                 const bool plain = !gf.codes;   // every cell fluid with in-grid ghosts
+                if constexpr (sizeof(T) > sizeof(C)) zs[t] = As[t] = ds[t] = rs[t] = (C)0;
                 if (!plain && is_solid(fs[t])) continue;
                 const C eP = R::get(ec, t);
                 const C xm = t == 0 ? left : R::get(ec, t - 1), xp = t == W - 1 ? right : R::get(ec, t + 1);
@@ -1391,23 +1393,44 @@ __device__ void FcgDotVK<TR, TZ, W, F>::run(const BlockAt& at) const {
                     A = A7_general<C>(L, fs[t], eP, xm, xp, ya, yb, za, zb);
                 }
                 const C d = R::get(dd, t), rv = RR::get(rr, t);
-                a0 = fma(eP, A, a0);
-                a1 = fma(A, d, a1);
-                a2 = fma(rv, eP, a2);
-                a3 = fma(rv, d, a3);
+                if constexpr (sizeof(T) > sizeof(C)) {
+                    zs[t] = eP;
+                    As[t] = A;
+                    ds[t] = d;
+                    rs[t] = rv;
+                } else {
+                    a0 = fma(eP, A, a0);
+                    a1 = fma(A, d, a1);
+                    a2 = fma(rv, eP, a2);
+                    a3 = fma(rv, d, a3);
+                }
+            }
+            if constexpr (sizeof(T) > sizeof(C)) {
+                T zt[W], At[W], dt[W], rt[W];
+                widened(zs, zt);
+                widened(As, At);
+                widened(ds, dt);
+                widened(rs, rt);
+#pragma unroll
+                for (int t = 0; t < W; ++t) {
+                    a0 = fma(zt[t], At[t], a0);
+                    a1 = fma(At[t], dt[t], a1);
+                    a2 = fma(rt[t], zt[t], a2);
+                    a3 = fma(rt[t], dt[t], a3);
+                }
             }
         }
         em = ec;
         ec = ep;
         ep = en;
     }
-    C s[4] = {a0, a1, a2, a3};   // (FP32 corrections: FP32 within a warp, FP64 from the warp sums on)
+    T s[4] = {a0, a1, a2, a3};
     fcg_reduce<kThreads>(s, partials, st, have, at);
 }
 
 // d = z - beta d_prev, p += alpha d (fluid cells), d kept: W consecutive
-// cells per thread, one-dimensional grid.  Needs N % W = 0.
-template <class TZ, int W>
+// cells per thread, one-dimensional grid, d and alpha d in T.  Needs N % W = 0.
+template <class TZ, int W, class T>
 struct FcgUpdVK {
     static constexpr int kThreads = 256;
     static constexpr bool kNoShared = true;   // run() uses no shared memory
@@ -1421,21 +1444,24 @@ struct FcgUpdVK {
         const int c = W * (at.b.x * kThreads + threadIdx.x);
         if (c >= L.N) return;
         using C = typename Acc<TZ>::type;
-        const C alpha = (C)st->g_alpha, beta = (C)st->g_beta;
+        const T alpha = (T)st->g_alpha, beta = (T)st->g_beta;
         C zv[W], dv[W];
 #pragma unroll
         for (int t = 0; t < W; ++t) dv[t] = (C)0;
         VecW<TZ, W>::load(z, c, zv);
-        if (beta != (C)0) VecW<TZ, W>::load_rw(dp, c, dv);
+        if (beta != (T)0) VecW<TZ, W>::load_rw(dp, c, dv);
         uint32_t fs[W];
         GroupFlags gf = {true, false, false};
         if constexpr (sizeof(C) == 4) gf = group_flags<W>(L.grp, c);
         const bool codes = gf.codes;
         if (codes) codes_w<W>(L.nbf, c, fs);
-        C d[W];
+        T d[W], zt[W];
+        widened(zv, zt);
+        widened(dv, d);
 #pragma unroll
-        for (int t = 0; t < W; ++t) d[t] = fma(-beta, dv[t], zv[t]);
-        VecW<TZ, W>::store(dp, c, d);
+        for (int t = 0; t < W; ++t) d[t] = fma(-beta, d[t], zt[t]);
+        narrowed(d, dv);
+        VecW<TZ, W>::store(dp, c, dv);
         if constexpr (sizeof(C) == 8) {
             double u[W];
             VecW<double, W>::load_rw(p, c, u);
@@ -1445,17 +1471,21 @@ struct FcgUpdVK {
             VecW<double, W>::store(p, c, u);
             return;
         }
+        float step[W];
+#pragma unroll
+        for (int t = 0; t < W; ++t) d[t] *= alpha;
+        narrowed(d, step);
         float4* pp = reinterpret_cast<float4*>(p + c);   // p as double-float pairs, two cells per 16 bytes
 #pragma unroll
         for (int h = 0; h < W / 2; ++h) {
             float4 u = pp[h];
             if (!codes || !is_solid(fs[2 * h])) {
-                const float2 x = pp_plus(make_float2(u.x, u.y), alpha * d[2 * h]);
+                const float2 x = pp_plus(make_float2(u.x, u.y), step[2 * h]);
                 u.x = x.x;
                 u.y = x.y;
             }
             if (!codes || !is_solid(fs[2 * h + 1])) {
-                const float2 x = pp_plus(make_float2(u.z, u.w), alpha * d[2 * h + 1]);
+                const float2 x = pp_plus(make_float2(u.z, u.w), step[2 * h + 1]);
                 u.z = x.x;
                 u.w = x.y;
             }
@@ -2252,49 +2282,40 @@ cudaError_t launch_prolong_add(int inner, const LevelDev& Lf, const LevelDev& Lc
     return err;
 }
 
-// z and the kept direction dp in TZ (the inner type, or FP32 on BF16 levels), r in TR
+// z and the kept direction dp in TZ (the inner type, or FP32 on BF16 levels), r in TR: W cells per
+// thread, products, sums and the step in T
+template <class TR, class TZ, int W, class T>
+static cudaError_t fcg_vector(const LevelDev& L, const TZ* z, const TR* r, TZ* dp, double* p, double* partials,
+                              SolveState* st, bool flags, cudaStream_t s) {
+    // (at most level0_blocks_max(n) blocks: partials has room)
+    int zc = 0;
+    const int lrl = vw_lrl(L.n[0], W);
+    const dim3 grid = vw_grid(L, W, lrl, zc);
+    cudaError_t err = cudaErrorInvalidValue;
+    if constexpr (sizeof(TZ) < 8)
+        if (flags) err = launch_k(FcgDotVK<TR, TZ, W, true, T>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s);
+    if (!flags) err = launch_k(FcgDotVK<TR, TZ, W, false, T>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s);
+    if (err != cudaSuccess) return err;
+    using U = FcgUpdVK<TZ, W, T>;
+    return launch_k(U{L, z, dp, p, st}, dim3((unsigned)((L.N / W + U::kThreads - 1) / U::kThreads)), dim3(U::kThreads), 0, s);
+}
+
 template <class TR, class TZ>
 static cudaError_t fcg_launch(const LevelDev& L, const TZ* z, const TR* r, TZ* dp, double* p, double* partials,
                               SolveState* st, cudaStream_t s) {
     if constexpr (sizeof(TR) < 8) {
-        // (whatever the size: the one-cell pair, with its sums in FP64, took 58 us at 430,080 cells;
-        // this and the float-float residual together brought ten steps of that room from 18.9 to
-        // 13.4 ms)
         if (L.n[0] % 4 == 0) {
-            // (at most level0_blocks_max(n) blocks: partials has room)
-            int zc = 0;
+            // products, sums, alpha and beta in FP32 on large levels and in batches; in FP64 on the smaller
+            // ones of a case alone (430,080 cells, us for the pair of launches: one cell per thread 58, this
+            // 35, the FP32 form 22)
+            if (L.N < (1 << 20) && !g_rec) return fcg_vector<TR, TZ, 4, double>(L, z, r, dp, p, partials, st, by_flags(L), s);
             constexpr int W = std::is_same<TR, TZ>::value ? vec_w<TR>() : 4;
-            if (W == 8 && L.n[0] % 8 == 0) {
-                const int lrl = vw_lrl(L.n[0], W);
-                const dim3 grid = vw_grid(L, W, lrl, zc);
-                cudaError_t err =
-                    by_flags(L) ? launch_k(FcgDotVK<TR, TZ, W, true>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s)
-                                : launch_k(FcgDotVK<TR, TZ, W, false>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s);
-                if (err != cudaSuccess) return err;
-                const unsigned nb = (unsigned)((L.N / W + FcgUpdVK<TZ, W>::kThreads - 1) / FcgUpdVK<TZ, W>::kThreads);
-                return launch_k(FcgUpdVK<TZ, W>{L, z, dp, p, st}, dim3(nb), dim3(FcgUpdVK<TZ, W>::kThreads), 0, s);
-            }
-            const int lrl = vw_lrl(L.n[0], 4);
-            const dim3 grid = vw_grid(L, 4, lrl, zc);
-            cudaError_t err =
-                by_flags(L) ? launch_k(FcgDotVK<TR, TZ, 4, true>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s)
-                            : launch_k(FcgDotVK<TR, TZ, 4, false>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s);
-            if (err != cudaSuccess) return err;
-            const unsigned nb = (unsigned)((L.N / 4 + FcgUpdVK<TZ, 4>::kThreads - 1) / FcgUpdVK<TZ, 4>::kThreads);
-            return launch_k(FcgUpdVK<TZ, 4>{L, z, dp, p, st}, dim3(nb), dim3(FcgUpdVK<TZ, 4>::kThreads), 0, s);
+            if (L.n[0] % W == 0) return fcg_vector<TR, TZ, W, float>(L, z, r, dp, p, partials, st, by_flags(L), s);
+            return fcg_vector<TR, TZ, 4, float>(L, z, r, dp, p, partials, st, by_flags(L), s);
         }
     }
     if constexpr (sizeof(TR) == 8) {
-        if (L.n[0] % 2 == 0) {
-            int zc = 0;
-            const int lrl = vw_lrl(L.n[0], 2);
-            const dim3 grid = vw_grid(L, 2, lrl, zc);
-            cudaError_t err =
-                launch_k(FcgDotVK<TR, TZ, 2, false>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s);
-            if (err != cudaSuccess) return err;
-            const unsigned nb = (unsigned)((L.N / 2 + FcgUpdVK<TZ, 2>::kThreads - 1) / FcgUpdVK<TZ, 2>::kThreads);
-            return launch_k(FcgUpdVK<TZ, 2>{L, z, dp, p, st}, dim3(nb), dim3(FcgUpdVK<TZ, 2>::kThreads), 0, s);
-        }
+        if (L.n[0] % 2 == 0) return fcg_vector<TR, TZ, 2, double>(L, z, r, dp, p, partials, st, false, s);
     }
     cudaError_t err = launch_k(FcgDotK<TR, TZ>{L, z, r, dp, partials, st}, grid3(L), kBlock3, 0, s);
     if (err != cudaSuccess) return err;
