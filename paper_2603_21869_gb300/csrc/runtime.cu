@@ -1559,6 +1559,7 @@ void free_batch(fvm_batch* b) {
 // Lay the merged launches' tables into one device buffer: per launch the
 // functor table, the block offsets, the per-case grids, and (resid0) the
 // block counter and the list of its cases' solve states.
+// (A residual launch's list holds every case's: the last launch of several decides for all.)
 fvm_status build_arena(std::vector<Merged>* segs, int nseg, const std::vector<fvm_case*>& cases, void** arena_out) {
     auto up = [](size_t x, size_t a) { return (x + a - 1) / a * a; };
     size_t bytes = 0;
@@ -1568,7 +1569,7 @@ fvm_status build_arena(std::vector<Merged>* segs, int nseg, const std::vector<fv
             bytes = up(bytes, 256) + n * m.recs[0]->arg.size();
             bytes = up(bytes, 16) + (n + 1) * sizeof(int);
             bytes = up(bytes, 16) + n * sizeof(uint3);
-            bytes = up(bytes, 16) + n * sizeof(SolveState*);
+            bytes = up(bytes, 16) + cases.size() * sizeof(SolveState*);
             bytes = up(bytes, 16) + 16;
         }
     bytes = up(bytes, 256);
@@ -1614,13 +1615,13 @@ fvm_status build_arena(std::vector<Merged>* segs, int nseg, const std::vector<fv
             off = up(off, 16);
             SolveState** lst = (SolveState**)&host[off];
             m.ctl.st = (SolveState* const*)(d + off);
-            for (size_t i = 0; i < n; ++i) lst[i] = cases[m.cases[i]]->sst;
-            off += n * sizeof(SolveState*);
+            for (size_t i = 0; i < cases.size(); ++i) lst[i] = cases[i]->sst;
+            off += cases.size() * sizeof(SolveState*);
             off = up(off, 16);
             m.ctl.counter = (unsigned*)(d + off);   // zero
             off += 16;
             m.map.n = (int)n;
-            m.ctl.n = (int)n;
+            m.ctl.n = (int)cases.size();
             if (tot >= ((int64_t)1 << 31)) {
                 cudaFree(dev);
                 return fail(FVM_ERR_INVALID, "batch too large for one launch");
@@ -1691,16 +1692,18 @@ fvm_status batch_capture(fvm_batch* B, fvm_batch::Graph& G) {
     if (st != FVM_OK) return st;
     std::vector<Merged>* seg = G.seg;
     for (int s = 0; s < 4; ++s) seg[s] = merge_sequences(rec[s]);
-    if (seg[1].size() != 1)
-        return fail(FVM_ERR_INVALID, "batched cases need the same precisions (one level-0 residual launch)");
+    // FP64 cases with a collapsed x axis have a residual kernel of their own; where the reduced-precision
+    // ones differ (x extents of whole quads or not) the batch is refused
+    if (seg[1].size() != 1 && B->cases[0]->inner != FVM_FP64)
+        return fail(FVM_ERR_INVALID, "batched FP32 or BF16 cases need x extents that are all multiples of 4, or none");
     ST_TRY(build_arena(seg, 4, B->cases, &G.arena));
     for (int s = 0; s < 4; ++s)
         for (Merged& m : seg[s]) m.recs.clear();   // the recorded functors now live in the arena
     // dynamic shared-memory limits of the batched kernels (outside the capture)
     for (int s = 0; s < 4; ++s)
         for (Merged& m : seg[s]) CUDA_TRY(m.many(m.tab, m.map, 0, m.block, m.smem, &m.ctl, B->stream));
-    G.per_step = (int64_t)(seg[0].size() + seg[3].size()) + 1 /* gather */ + 1 /* last residual */;
-    G.per_outer = 1 + (int64_t)seg[2].size();
+    G.per_step = (int64_t)(seg[0].size() + seg[3].size()) + 1 /* gather */ + (int64_t)seg[1].size() /* last residual */;
+    G.per_outer = (int64_t)(seg[1].size() + seg[2].size());
     cudaStream_t s = B->stream;
     if (!B->side) CUDA_TRY(cudaStreamCreateWithFlags(&B->side, cudaStreamNonBlocking));
     CUDA_TRY(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
@@ -1714,8 +1717,8 @@ fvm_status batch_capture(fvm_batch* B, fvm_batch::Graph& G) {
     if ((st = issue(seg[0], s)) != FVM_OK) return abort_capture(st);
     WhileCapture W;
     if ((st = W.create(s)) != FVM_OK) return abort_capture(st);
-    seg[1][0].ctl.cond = W.handle;
-    seg[1][0].ctl.use_cond = 1;
+    seg[1].back().ctl.cond = W.handle;
+    seg[1].back().ctl.use_cond = 1;
     if ((st = issue(seg[1], s)) != FVM_OK || (st = W.add(s)) != FVM_OK) return abort_capture(st);
     if (cudaStreamBeginCaptureToGraph(B->side, W.body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) !=
         cudaSuccess)
@@ -2498,7 +2501,8 @@ fvm_status fvm_batch_profile(fvm_batch* B, int32_t nsteps, fvm_kernel_stat* out,
         for (const Merged& m : G.seg[0])
             if (st == FVM_OK) st = run(m);
         for (int it = 0; st == FVM_OK; ++it) {
-            st = run(G.seg[1][0]);
+            for (const Merged& m : G.seg[1])
+                if (st == FVM_OK) st = run(m);
             if (st != FVM_OK) break;
             k_batch_gather<<<1, 256, 0, s>>>(B->d_sts, B->d_dts, B->d_gather, n, B->d_scratch);
             if (cudaMemcpyAsync(B->h_gather, B->d_gather, n * sizeof(BatchGather), cudaMemcpyDeviceToHost, s) !=
