@@ -754,7 +754,9 @@ __global__ void __launch_bounds__(kCtaThreads, 1) k_coarse_many(const CoarseK<TI
     __shared__ Slab<typename Acc<TI>::type> tab[FVM_MAX_LEVELS];
     const Body<TI> b(k, g_coarse_smem, tab, block_rank(S));
     b.prologue();
-    pdl_enter();
+    // (the next kernel starts when this one ends: its blocks, let in early, kept the last clusters from
+    // finding their blocks' shared memory, 250 us a V-cycle with 64 cases; eight cases lose 0.5 %)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (k.st->active == 0) return;   // a converged case: its whole cluster leaves
     b.run();
 }
@@ -896,13 +898,12 @@ static int64_t cells_per_block(int inner, int S) {
 }
 constexpr size_t kSmemBudget = 222 * 1024;   // (227 KB less the static arrays)
 
-static bool plan_from(const std::vector<LevelDev>& levels, const std::vector<uint32_t>& dir, int inner, int S, int lc,
+bool coarse_plan_from(const std::vector<LevelDev>& levels, const std::vector<uint32_t>& dir, int inner, int S, int lc,
                       CoarsePlan& pl) {
     memset((void*)&pl, 0, sizeof(pl));
     pl.S = S;
     pl.lc = lc;
     pl.nl = (int)levels.size() - lc;
-    if (levels[lc].N > cells_per_block(inner, S) * S && pl.nl > 1) return false;
     const size_t cs = inner == FVM_FP64 ? 8 : 4;
     for (int top_global = 0; top_global < 2; ++top_global) {
         size_t q = 0, codes = 0;
@@ -963,13 +964,16 @@ bool coarse_plan(const std::vector<LevelDev>& levels, const std::vector<uint32_t
         if (!quads && v.N > cells_per_block(inner, S) * S / (inner == FVM_FP64 ? 2 : 4)) first = 1;
     }
     for (int lc = first; lc < (int)levels.size(); ++lc) {
-        if (!plan_from(levels, dir, inner, S, lc, pl)) continue;
+        if (levels[lc].N > cells_per_block(inner, S) * S && lc + 1 < (int)levels.size()) continue;
+        if (!coarse_plan_from(levels, dir, inner, S, lc, pl)) continue;
         if (exact || S == 1 || pl.lm > 0 || pl.nl == 1) return true;
-        return plan_from(levels, dir, inner, 1, lc, pl) || plan_from(levels, dir, inner, S, lc, pl);
+        return coarse_plan_from(levels, dir, inner, 1, lc, pl) || coarse_plan_from(levels, dir, inner, S, lc, pl);
     }
     return false;
 }
 
+// (the results are those of any number of blocks from the same finest level: only who works on a
+// cell changes, not its arithmetic)
 int coarse_cluster_for(int cases) {
     for (int S : {16, 8, 4, 2})
         if (cases * S <= (S == 16 ? 112 : 144)) return S;

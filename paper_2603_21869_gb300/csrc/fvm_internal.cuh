@@ -172,7 +172,7 @@ struct LevelDev {
                              // z), 2 / 4 the first cell's x- / the last cell's x+ face is a zero-value
                              // domain face.  Where 1 is clear every ghost is the load clamped into the
                              // grid, along x with that sign.
-    int32_t solids, pad;     // the level has solid cells
+    int32_t solids, level;   // the level has solid cells; its number
 };
 
 // Device-side state of one pressure solve: the last residual norms and the
@@ -373,6 +373,9 @@ cudaError_t launch_prolong_add(int inner, const LevelDev& Lf, const LevelDev& Lc
 // finest level that may be among them
 bool coarse_plan(const std::vector<LevelDev>& levels, const std::vector<uint32_t>& dir, int inner, int S, bool exact,
                  int first, CoarsePlan& pl);
+// the plan of a cluster of S blocks from level lc on, whatever its size; false where it does not fit
+bool coarse_plan_from(const std::vector<LevelDev>& levels, const std::vector<uint32_t>& dir, int inner, int S, int lc,
+                      CoarsePlan& pl);
 int coarse_cluster_for(int cases);   // blocks per cluster when this many cases run theirs at once
 // sets the kernel's limits; an error where the device cannot run such a cluster
 cudaError_t prepare_coarse(int inner, const CoarsePlan& pl);
@@ -629,7 +632,7 @@ struct Recorder {
     std::string site;                  // set by the caller before each launch site
     double bytes = 0.0;                // algorithmic bytes of the site (given to its first launch)
     int cases = 1;                     // cases of the batch being recorded
-    bool solids = false;               // some of them have solid cells
+    uint32_t solids = 0, clear = 0;    // bit l: some of them have a level l with / without solid cells
 };
 
 extern thread_local Recorder* g_rec;

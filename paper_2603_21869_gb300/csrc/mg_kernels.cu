@@ -572,8 +572,23 @@ template <int W> __device__ __forceinline__ GroupFlags group_flags(const uint8_t
 // second, dependent load for some groups of most warps costs a room more than the bytes: 512 x 256
 // x 128 cells, BF16: residual 104 us with the codes, 109 with the flags; residual and restriction 42
 // and 45; inner products and update 141 and 144 (512 x 128 x 128 FP32 channel: 66 and 59, 30 and
-// 25.5, 80 and 67 us, the other way round).
-static bool by_flags(const LevelDev& L) { return g_rec ? !g_rec->solids : !L.solids; }
+// 25.5, 80 and 67 us, the other way round).  The two round a cell at a zero-value x face differently,
+// so a batch with both kinds of level takes the third form, which chooses by the level: a case's
+// results do not depend on the other cases (inner products of eight served cases 53 us, by the
+// codes throughout 46).
+enum { kCodes = 0, kFlags = 1, kByLevel = 2 };
+template <int F> __device__ __forceinline__ bool takes_flags(const LevelDev& L) {
+    return F == kFlags || (F == kByLevel && !L.solids);
+}
+// go(form) with the form as a compile-time constant
+template <class Go>
+static cudaError_t by_form(const LevelDev& L, Go go) {
+    const bool solids = g_rec ? (g_rec->solids >> L.level) & 1u : L.solids != 0;
+    const bool clear = g_rec ? (g_rec->clear >> L.level) & 1u : L.solids == 0;
+    if (solids && clear) return go(std::integral_constant<int, kByLevel>());
+    if (solids) return go(std::integral_constant<int, kCodes>());
+    return go(std::integral_constant<int, kFlags>());
+}
 
 // cells per thread of the vector kernels on a level of this storage type
 template <class TI> __device__ __host__ constexpr int vec_w() { return sizeof(TI) == 2 ? 8 : (sizeof(TI) == 4 ? 4 : 2); }
@@ -1041,7 +1056,7 @@ __device__ __forceinline__ int resid0_sums(double s0, double s1, double* partial
 
 // r = b - A p (float-float), r^2 and b^2, the first pre-sweep e = w_J r / D;
 // four x cells per thread and a z march (the sweep's layout).  FP32 b, nx % 4 = 0.
-template <class TI, bool F>   // F: by the group flags
+template <class TI, int F>   // F: kCodes, kFlags or kByLevel
 struct Resid0V4K {
     static constexpr int kThreads = TX * TY;
     static constexpr int kMinBlocks = 3;       // at most 80 registers
@@ -1061,7 +1076,7 @@ struct Resid0V4K {
     __device__ int run(const BlockAt& at) const;
 };
 
-template <class TI, bool F>
+template <class TI, int F>
 __device__ int Resid0V4K<TI, F>::run(const BlockAt& at) const {
     const int nx = L.n[0], ny = L.n[1], nz = L.n[2];
     const int LR = 1 << lrl, lane = threadIdx.x & (LR - 1), sub = threadIdx.x >> lrl;
@@ -1079,6 +1094,7 @@ __device__ int Resid0V4K<TI, F>::run(const BlockAt& at) const {
     const float wJ = LP<float>::wJ(L), iD = LP<float>::iD(L);
     const double* const pp = this->p;
     const uint16_t* const nbf = L.nbf;
+    const bool flags = takes_flags<F>(L);
     FF em[4], ec[4], ep[4];
     ff_load4(pp, max(k0 - 1, 0) * sz + own, em);
     ff_load4(pp, k0 * sz + own, ec);
@@ -1091,7 +1107,7 @@ __device__ int Resid0V4K<TI, F>::run(const BlockAt& at) const {
         ff_load4(pp, base + op, yp);
         const float4 bq = __ldg(reinterpret_cast<const float4*>(b + base + own));
         GroupFlags gf = {true, false, false};
-        if constexpr (F) gf = group_flags<4>(L.grp, base + own);
+        if (flags) gf = group_flags<4>(L.grp, base + own);
         uint32_t fs[4] = {0u, 0u, 0u, 0u};
         if (gf.codes) codes_w<4>(nbf, base + own, fs);
         const FF xls = lane == 0 ? pp_load(pp, base + xl) : FF{0.0f, 0.0f};
@@ -1102,21 +1118,21 @@ __device__ int Resid0V4K<TI, F>::run(const BlockAt& at) const {
             l2_prefetch(pp + fb);
             l2_prefetch(pp + fb + 2);
             l2_prefetch(b + fb);
-            if constexpr (!F) l2_prefetch(nbf + fb);
+            if (!flags) l2_prefetch(nbf + fb);
         }
         if (k + 1 < k1) {   // the next plane's rows into L1 (their loads open the next iteration)
             const int nb = (k + 1) * sz;
             l1_prefetch(pp + nb + om);
             l1_prefetch(pp + nb + op);
             l1_prefetch(b + nb + own);
-            if constexpr (!F) l1_prefetch(nbf + nb + own);
+            if (!flags) l1_prefetch(nbf + nb + own);
         }
         FF left = {__shfl_up_sync(0xffffffffu, ec[3].h, 1, LR), __shfl_up_sync(0xffffffffu, ec[3].l, 1, LR)};
         FF right = {__shfl_down_sync(0xffffffffu, ec[0].h, 1, LR), __shfl_down_sync(0xffffffffu, ec[0].l, 1, LR)};
         if (lane == 0) left = xls;
         if (lane == LR - 1) right = xrs;
         if (lastc) right = ec[3];
-        if constexpr (F) {   // (at a row's ends left / right is the cell itself)
+        if constexpr (F != kCodes) {   // (at a row's ends left / right is the cell itself)
             if (gf.neg_l) left = ff_neg(left);
             if (gf.neg_r) right = ff_neg(right);
         }
@@ -1287,7 +1303,7 @@ __device__ int Resid0DK<TB, TI>::run(const BlockAt& at) const {
 // (the sweep's layout and neighbour scheme): products, the thread's and the
 // warp's sums in T, block and grid sums in FP64.  Needs nx % W = 0.
 // (TR: storage of r; TZ: storage of z and the kept direction, FP32 on BF16 levels)
-template <class TR, class TZ, int W, bool F, class T>   // F: by the group flags
+template <class TR, class TZ, int W, int F, class T>   // F: kCodes, kFlags or kByLevel
 struct FcgDotVK {
     static constexpr int kThreads = TX * TY;
     static constexpr int kMinBlocks = sizeof(T) > sizeof(TZ) ? 3 : 4;   // at most 64 registers (FP64 sums of FP32 fields: 80)
@@ -1304,7 +1320,7 @@ struct FcgDotVK {
     __device__ void run(const BlockAt& at) const;
 };
 
-template <class TR, class TZ, int W, bool F, class T>
+template <class TR, class TZ, int W, int F, class T>
 __device__ void FcgDotVK<TR, TZ, W, F, T>::run(const BlockAt& at) const {
     using C = typename Acc<TZ>::type;
     using R = RawW<TZ, W>;
@@ -1324,6 +1340,7 @@ __device__ void FcgDotVK<TR, TZ, W, F, T>::run(const BlockAt& at) const {
     const bool have = st->g_valid != 0;
     const TZ* const zz = this->z;
     const uint16_t* const nbf = L.nbf;
+    const bool flags = takes_flags<F>(L);
     typename R::T em = R::load(zz, max(k0 - 1, 0) * sz + own);
     typename R::T ec = R::load(zz, k0 * sz + own);
     typename R::T ep = R::load(zz, min(k0 + 1, nz - 1) * sz + own);
@@ -1337,7 +1354,7 @@ __device__ void FcgDotVK<TR, TZ, W, F, T>::run(const BlockAt& at) const {
         if (have) dd = R::load(dp, base + own);
         uint32_t fs[W];
         GroupFlags gf = {true, false, false};
-        if constexpr (F) gf = group_flags<W>(L.grp, base + own);
+        if (flags) gf = group_flags<W>(L.grp, base + own);
         if (gf.codes) codes_w<W>(nbf, base + own, fs);
         const C xls = lane == 0 ? to_c<C>(ldg(zz + base + xl)) : (C)0;
         const C xrs = lane == LR - 1 ? to_c<C>(ldg(zz + base + xr)) : (C)0;
@@ -1346,7 +1363,7 @@ __device__ void FcgDotVK<TR, TZ, W, F, T>::run(const BlockAt& at) const {
             const int fb = (k + 3) * sz + own;
             l2_prefetch(zz + fb);
             l2_prefetch(r + fb);
-            if constexpr (!F) l2_prefetch(nbf + fb);
+            if (!flags) l2_prefetch(nbf + fb);
             if (have) l2_prefetch(dp + fb);
         }
         if (k + 1 < k1) {   // the next plane's rows into L1 (their loads open the next iteration)
@@ -1354,7 +1371,7 @@ __device__ void FcgDotVK<TR, TZ, W, F, T>::run(const BlockAt& at) const {
             l1_prefetch(zz + nb + om);
             l1_prefetch(zz + nb + op);
             l1_prefetch(r + nb + own);
-            if constexpr (!F) l1_prefetch(nbf + nb + own);
+            if (!flags) l1_prefetch(nbf + nb + own);
             if (have) l1_prefetch(dp + nb + own);
         }
         C left = __shfl_up_sync(0xffffffffu, R::get(ec, W - 1), 1, LR);
@@ -1362,7 +1379,7 @@ __device__ void FcgDotVK<TR, TZ, W, F, T>::run(const BlockAt& at) const {
         if (lane == 0) left = xls;
         if (lane == LR - 1) right = xrs;
         if (lastc) right = R::get(ec, W - 1);
-        if constexpr (F) {   // (at a row's ends left / right is the cell itself)
+        if (flags) {   // (at a row's ends left / right is the cell itself)
             if (gf.neg_l) left = -left;
             if (gf.neg_r) right = -right;
         } else {
@@ -1469,27 +1486,27 @@ struct FcgUpdVK {
             for (int t = 0; t < W; ++t)
                 if (!is_solid(fs[t])) u[t] = fma(alpha, d[t], u[t]);
             VecW<double, W>::store(p, c, u);
-            return;
-        }
-        float step[W];
+        } else {
+            float step[W];
 #pragma unroll
-        for (int t = 0; t < W; ++t) d[t] *= alpha;
-        narrowed(d, step);
-        float4* pp = reinterpret_cast<float4*>(p + c);   // p as double-float pairs, two cells per 16 bytes
+            for (int t = 0; t < W; ++t) d[t] *= alpha;
+            narrowed(d, step);
+            float4* pp = reinterpret_cast<float4*>(p + c);   // p as double-float pairs, two cells per 16 bytes
 #pragma unroll
-        for (int h = 0; h < W / 2; ++h) {
-            float4 u = pp[h];
-            if (!codes || !is_solid(fs[2 * h])) {
-                const float2 x = pp_plus(make_float2(u.x, u.y), step[2 * h]);
-                u.x = x.x;
-                u.y = x.y;
+            for (int h = 0; h < W / 2; ++h) {
+                float4 u = pp[h];
+                if (!codes || !is_solid(fs[2 * h])) {
+                    const float2 x = pp_plus(make_float2(u.x, u.y), step[2 * h]);
+                    u.x = x.x;
+                    u.y = x.y;
+                }
+                if (!codes || !is_solid(fs[2 * h + 1])) {
+                    const float2 x = pp_plus(make_float2(u.z, u.w), step[2 * h + 1]);
+                    u.z = x.x;
+                    u.w = x.y;
+                }
+                pp[h] = u;
             }
-            if (!codes || !is_solid(fs[2 * h + 1])) {
-                const float2 x = pp_plus(make_float2(u.z, u.w), step[2 * h + 1]);
-                u.z = x.x;
-                u.w = x.y;
-            }
-            pp[h] = u;
         }
     }
 };
@@ -1626,7 +1643,7 @@ __device__ void ProlongVK<TI, W>::run(const BlockAt& at) const {
 // writes the W/2 coarse cells I0 = i4/2 .. (mean of their children's r - A e,
 // Eq. restriction).  Rows j +- 1 and planes k +- 1 are loaded whole, x
 // neighbours by shuffles.  Needs x and y active, nx % W = 0, ny even.
-template <class TI, int W, bool F>   // F: by the group flags
+template <class TI, int W, int F>   // F: kCodes, kFlags or kByLevel
 struct RRVK {
     static constexpr int kThreads = TX * TY;
     static constexpr bool kNoShared = true;   // run() uses no shared memory
@@ -1642,7 +1659,7 @@ struct RRVK {
     __device__ void run(const BlockAt& at) const;
 };
 
-template <class TI, int W, bool F>
+template <class TI, int W, int F>
 __device__ void RRVK<TI, W, F>::run(const BlockAt& at) const {
     using C = typename Acc<TI>::type;
     using R = RawW<TI, W>;
@@ -1662,6 +1679,7 @@ __device__ void RRVK<TI, W, F>::run(const BlockAt& at) const {
     const TI* const ep = e;
     const TI* const rp = r;
     const uint16_t* const nbf = Lf.nbf;
+    const bool flags = takes_flags<F>(Lf);
     auto at_ = [&](int jj, int kk) { return ic + sy * jj + sz * kk; };
     C s[H];   // sums of the coarse cells I0 .. I0 + H - 1
 #pragma unroll
@@ -1680,7 +1698,7 @@ __device__ void RRVK<TI, W, F>::run(const BlockAt& at) const {
             const typename R::T rr = R::load(rp, at_(jr, k));
             uint32_t fs[W];
             GroupFlags gf = {true, false, false};
-            if constexpr (F) gf = group_flags<W>(Lf.grp, at_(jr, k));
+            if (flags) gf = group_flags<W>(Lf.grp, at_(jr, k));
             if (gf.codes) codes_w<W>(nbf, at_(jr, k), fs);
             const C lx = lane == 0 ? to_c<C>(ldg(ep + max(ic - 1, 0) + sy * jr + sz * k)) : (C)0;
             const C rx = lane == LR - 1 ? to_c<C>(ldg(ep + min(ic + W, nx - 1) + sy * jr + sz * k)) : (C)0;
@@ -1689,13 +1707,13 @@ __device__ void RRVK<TI, W, F>::run(const BlockAt& at) const {
             if (lane == 0) left = lx;
             if (lane == LR - 1) right = rx;
             if (last) right = R::get(ec, W - 1);
-            if constexpr (F) {   // (at a row's ends left / right is the cell itself)
+            if constexpr (F != kCodes) {   // (at a row's ends left / right is the cell itself)
                 if (gf.neg_l) left = -left;
                 if (gf.neg_r) right = -right;
             }
 #pragma unroll
             for (int t = 0; t < W; ++t) {
-                if ((!F || gf.codes) && is_solid(fs[t])) continue;
+                if ((F == kCodes || gf.codes) && is_solid(fs[t])) continue;
                 const C eP = R::get(ec, t);
                 const C xm = t == 0 ? left : R::get(ec, t - 1), xp = t == W - 1 ? right : R::get(ec, t + 1);
                 const C ya = R::get(yl, t), yb = R::get(yh, t), za = R::get(zl, t), zb = R::get(zh, t);
@@ -1704,7 +1722,7 @@ __device__ void RRVK<TI, W, F>::run(const BlockAt& at) const {
                     continue;
                 }
                 C A;
-                if ((F && !gf.codes) || !((fs[t] >> 13) & 1u)) {
+                if ((F != kCodes && !gf.codes) || !((fs[t] >> 13) & 1u)) {
                     C sa = (xm + xp) * ihx;
                     sa = fma(ya + yb, ihy, sa);
                     sa = fma(za + zb, ihz, sa);
@@ -2044,17 +2062,16 @@ cudaError_t launch_solve_begin(SolveState* st, cudaStream_t s) {
     return launch_k(SolveBeginK{st}, dim3(1), dim3(1), 0, s);
 }
 
-static int sweep_planes(int tiles, int nz, int fixed, int per_sm, int W);
+static int sweep_planes(int tiles, int nz, int fixed, int per_sm, int W, bool sums);
 
 // vector kernels: the block's x-y extent for W cells per thread and the row segments of lrl;
-// per_sm: the blocks per SM the plane rule aims for
-static dim3 vw_grid(const LevelDev& L, int W, int lrl, int& zc, int per_sm = 8) {
+// per_sm: the blocks per SM the plane rule aims for; sums: the columns order a sum
+static dim3 vw_grid(const LevelDev& L, int W, int lrl, int& zc, int per_sm = 8, bool sums = false) {
     const int wx = W << lrl, wy = TY << (5 - lrl);
     const int tiles = ((L.n[0] + wx - 1) / wx) * ((L.n[1] + wy - 1) / wy);
-    zc = sweep_planes(tiles, L.n[2], L.zc_fixed, per_sm, W);
+    zc = sweep_planes(tiles, L.n[2], L.zc_fixed, per_sm, W, sums);
     return dim3((unsigned)((L.n[0] + wx - 1) / wx), (unsigned)((L.n[1] + wy - 1) / wy), (unsigned)((L.n[2] + zc - 1) / zc));
 }
-static dim3 v4_grid(const LevelDev& L, int lrl, int& zc) { return vw_grid(L, 4, lrl, zc); }
 
 cudaError_t launch_resid0(int inner, int bprec, const LevelDev& L, const double* p, const void* b, void* r, void* e,
                           double* partials, SolveState* st, cudaGraphConditionalHandle cond, int use_cond,
@@ -2066,13 +2083,12 @@ cudaError_t launch_resid0(int inner, int bprec, const LevelDev& L, const double*
             if (bprec == FVM_FP32 && L.n[0] % 4 == 0 && (L.N >= (1 << 20) || g_rec)) {
                 const int lrl = v4_lrl(L.n[0]);
                 int zc = 0;
-                const dim3 grid = v4_grid(L, lrl, zc);
+                const dim3 grid = vw_grid(L, 4, lrl, zc, 8, true);
                 // (at most level0_blocks_max(n) blocks: partials has room)
-                if (by_flags(L))
-                    return launch_r0(Resid0V4K<TI, true>{L, p, (const float*)b, (TI*)r, (TI*)e, partials, st, zc, lrl},
+                return by_form(L, [&](auto f) {
+                    return launch_r0(Resid0V4K<TI, decltype(f)::value>{L, p, (const float*)b, (TI*)r, (TI*)e, partials, st, zc, lrl},
                                      grid, dim3(TX, TY), cond, use_cond, s);
-                return launch_r0(Resid0V4K<TI, false>{L, p, (const float*)b, (TI*)r, (TI*)e, partials, st, zc, lrl}, grid,
-                                 dim3(TX, TY), cond, use_cond, s);
+                });
             }
         }
         // two cells per thread in FP64 on FP64 levels, and on the smaller ones of a reduced-precision
@@ -2081,7 +2097,7 @@ cudaError_t launch_resid0(int inner, int bprec, const LevelDev& L, const double*
         if (bprec == (sizeof(TI) == 8 ? FVM_FP64 : FVM_FP32) && L.n[0] % (sizeof(TI) == 8 ? 2 : 4) == 0) {
             const int lrl = vw_lrl(L.n[0], 2);
             int zc = 0;
-            const dim3 grid = vw_grid(L, 2, lrl, zc);
+            const dim3 grid = vw_grid(L, 2, lrl, zc, 8, true);
             return launch_r0(Resid0DK<TB, TI>{L, p, (const TB*)b, (TI*)r, (TI*)e, partials, st, zc, lrl}, grid,
                              dim3(TX, TY), cond, use_cond, s);
         }
@@ -2118,22 +2134,24 @@ static dim3 walk_grid(const LevelDev& L, int kz) {
 // one 12.94 -> 12.84 ms from four planes to eight; 24 cycles of a 256 x 128 x 128 BF16 room 5.70
 // -> 5.60 ms from two planes to four; the 512 x 256 x 128 room at 16 planes instead of 8 54.3 ->
 // 55.1 ms; at two, both kernels a third slower).
-static int sweep_planes(int tiles, int nz, int fixed, int per_sm, int W) {
+static int sweep_planes(int tiles, int nz, int fixed, int per_sm, int W, bool sums) {
     if (fixed > 0) return fixed < nz ? fixed : nz;
     auto blocks = [&](int zc) { return tiles * ((nz + zc - 1) / zc); };
+    const bool reduces = per_sm <= 8;
     if (g_rec) {
         // in a batch the cases' blocks add up (taken as all of this case's size): the longest columns
         // of at most eight planes that leave the launch this many blocks, fewer for the kernels that
         // end in a block reduction and more for the eight-cell sweep (two planes of a small level's
         // block take longer than the level: with eight-plane columns throughout, 8 FP32 channels
         // took 14.8 ms for four steps against 13.6 ms, 8 served BF16 cases 43.9 against 34.0 ms for
-        // two; 64 channels 19.4 ms a step either way)
-        const int want = per_sm <= 8 ? 300 : (W == 8 ? 1500 : 608);
+        // two; 64 channels 19.4 ms a step either way).  Columns that order a sum are those of a batch of
+        // eight in any batch (as of four, the residual of 8 channels took 77 us for 63): a case's
+        // results do not depend on how many others there are
+        const int want = reduces ? 300 : (W == 8 ? 1500 : 608);
         for (int zc : {8, 4, 2})
-            if ((int64_t)blocks(zc) * g_rec->cases >= want) return nz < zc ? nz : zc;
+            if ((int64_t)blocks(zc) * (sums ? 8 : g_rec->cases) >= want) return nz < zc ? nz : zc;
         return 1;
     }
-    const bool reduces = per_sm <= 8;
     for (int zc : {32, 16, 8, 4, 2})
         if (blocks(zc) >= (reduces && zc <= 8 ? 1000 : per_sm * 152)) return zc;
     return reduces && blocks(2) >= 2 * 152 ? 2 : 1;
@@ -2219,18 +2237,15 @@ cudaError_t launch_resid_restrict(int inner, const LevelDev& Lf, const LevelDev&
         };
         using W4 = std::integral_constant<int, 4>;
         using W8 = std::integral_constant<int, 8>;
-        using Yes = std::true_type;
-        using No = std::false_type;
-        const bool f = by_flags(Lf);
-        if (inner == FVM_FP32) return f ? go(0.0f, W4(), Yes()) : go(0.0f, W4(), No());
+        if (inner == FVM_FP32) return by_form(Lf, [&](auto f) { return go(0.0f, W4(), f); });
         const __nv_bfloat16 b16{};
-        if (W == 8) return f ? go(b16, W8(), Yes()) : go(b16, W8(), No());
-        return f ? go(b16, W4(), Yes()) : go(b16, W4(), No());
+        if (W == 8) return by_form(Lf, [&](auto f) { return go(b16, W8(), f); });
+        return by_form(Lf, [&](auto f) { return go(b16, W4(), f); });
     }
     if (inner == FVM_FP64 && Lf.active[0] && Lf.active[1]) {   // (active axes of a level that is coarsened are even)
         const int lrl = vw_lrl(Lf.n[0], 2), wx = 2 << lrl, wy = TY << (5 - lrl);
         const dim3 grid((unsigned)((Lf.n[0] + wx - 1) / wx), (unsigned)((Lc.n[1] + wy - 1) / wy), (unsigned)Lc.n[2]);
-        return launch_k(RRVK<double, 2, false>{Lf, Lc, (const double*)e, (const double*)r, (double*)rc, (double*)ec0, lrl, st},
+        return launch_k(RRVK<double, 2, kCodes>{Lf, Lc, (const double*)e, (const double*)r, (double*)rc, (double*)ec0, lrl, st},
                         grid, dim3(TX, TY), 0, s);
     }
     if (Lf.active[0] && Lf.active[1]) {
@@ -2286,15 +2301,17 @@ cudaError_t launch_prolong_add(int inner, const LevelDev& Lf, const LevelDev& Lc
 // thread, products, sums and the step in T
 template <class TR, class TZ, int W, class T>
 static cudaError_t fcg_vector(const LevelDev& L, const TZ* z, const TR* r, TZ* dp, double* p, double* partials,
-                              SolveState* st, bool flags, cudaStream_t s) {
+                              SolveState* st, cudaStream_t s) {
     // (at most level0_blocks_max(n) blocks: partials has room)
     int zc = 0;
     const int lrl = vw_lrl(L.n[0], W);
-    const dim3 grid = vw_grid(L, W, lrl, zc);
-    cudaError_t err = cudaErrorInvalidValue;
-    if constexpr (sizeof(TZ) < 8)
-        if (flags) err = launch_k(FcgDotVK<TR, TZ, W, true, T>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s);
-    if (!flags) err = launch_k(FcgDotVK<TR, TZ, W, false, T>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s);
+    const dim3 grid = vw_grid(L, W, lrl, zc, 8, true);
+    auto dot = [&](auto f) {
+        return launch_k(FcgDotVK<TR, TZ, W, decltype(f)::value, T>{L, z, r, dp, partials, st, zc, lrl}, grid, dim3(TX, TY), 0, s);
+    };
+    cudaError_t err;
+    if constexpr (sizeof(TZ) == 8) err = dot(std::integral_constant<int, kCodes>());
+    else err = by_form(L, dot);
     if (err != cudaSuccess) return err;
     using U = FcgUpdVK<TZ, W, T>;
     return launch_k(U{L, z, dp, p, st}, dim3((unsigned)((L.N / W + U::kThreads - 1) / U::kThreads)), dim3(U::kThreads), 0, s);
@@ -2308,14 +2325,14 @@ static cudaError_t fcg_launch(const LevelDev& L, const TZ* z, const TR* r, TZ* d
             // products, sums, alpha and beta in FP32 on large levels and in batches; in FP64 on the smaller
             // ones of a case alone (430,080 cells, us for the pair of launches: one cell per thread 58, this
             // 35, the FP32 form 22)
-            if (L.N < (1 << 20) && !g_rec) return fcg_vector<TR, TZ, 4, double>(L, z, r, dp, p, partials, st, by_flags(L), s);
+            if (L.N < (1 << 20) && !g_rec) return fcg_vector<TR, TZ, 4, double>(L, z, r, dp, p, partials, st, s);
             constexpr int W = std::is_same<TR, TZ>::value ? vec_w<TR>() : 4;
-            if (L.n[0] % W == 0) return fcg_vector<TR, TZ, W, float>(L, z, r, dp, p, partials, st, by_flags(L), s);
-            return fcg_vector<TR, TZ, 4, float>(L, z, r, dp, p, partials, st, by_flags(L), s);
+            if (L.n[0] % W == 0) return fcg_vector<TR, TZ, W, float>(L, z, r, dp, p, partials, st, s);
+            return fcg_vector<TR, TZ, 4, float>(L, z, r, dp, p, partials, st, s);
         }
     }
     if constexpr (sizeof(TR) == 8) {
-        if (L.n[0] % 2 == 0) return fcg_vector<TR, TZ, 2, double>(L, z, r, dp, p, partials, st, false, s);
+        if (L.n[0] % 2 == 0) return fcg_vector<TR, TZ, 2, double>(L, z, r, dp, p, partials, st, s);
     }
     cudaError_t err = launch_k(FcgDotK<TR, TZ>{L, z, r, dp, partials, st}, grid3(L), kBlock3, 0, s);
     if (err != cudaSuccess) return err;
