@@ -987,6 +987,13 @@ cudaError_t prepare_coarse(int inner, const CoarsePlan& pl) {
     return prepare_kernel(fn, pl.S, pl.smem);
 }
 
+cudaError_t prepare_coarse_many(int inner, int S, size_t smem) {
+    const void* fn = inner == FVM_FP64   ? (const void*)k_coarse_many<double>
+                     : inner == FVM_FP32 ? (const void*)k_coarse_many<float>
+                                         : (const void*)k_coarse_many<__nv_bfloat16>;
+    return prepare_kernel(fn, S, smem);
+}
+
 cudaError_t launch_coarse(int inner, const CoarsePlan& pl, const void* r_in, void* e_out, double* p,
                           const double* Ainv, const SolveState* st, cudaStream_t s) {
     if (inner == FVM_FP64) return launch<double>(pl, r_in, e_out, p, Ainv, st, s);

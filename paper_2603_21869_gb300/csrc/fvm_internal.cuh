@@ -379,6 +379,7 @@ bool coarse_plan_from(const std::vector<LevelDev>& levels, const std::vector<uin
 int coarse_cluster_for(int cases);   // blocks per cluster when this many cases run theirs at once
 // sets the kernel's limits; an error where the device cannot run such a cluster
 cudaError_t prepare_coarse(int inner, const CoarsePlan& pl);
+cudaError_t prepare_coarse_many(int inner, int S, size_t smem);   // the same for a batch's kernel
 // flexible CG with one kept direction around the V-cycles: the inner products
 // of z (the V-cycles' correction) with A z, r and the kept direction d_prev
 // (last block: beta, alpha), then d = z - beta d_prev, p += alpha d, d kept.

@@ -17,6 +17,7 @@
 #include <thread>
 #include <vector>
 
+#include "cluster_rule.h"
 #include "fvm_internal.cuh"
 #include "host_buffer.h"
 
@@ -1153,24 +1154,31 @@ bool plan_coarse_levels(const fvm_case* c, int S, bool exact, CoarsePlan& cp) {
 // number of cases: a case's results are the same in every batch), in clusters of as many blocks as
 // there is room for all of them at once, or the next size that holds the levels.  From what 8 blocks
 // take, batches of two to five served cases were 2-12 % slower, of 20 to 64 channels as fast.
+// (On a device that holds no such cluster the line is the largest one's that it does hold.)
 fvm_status plan_batch_coarse(const std::vector<fvm_case*>& cases) {
     constexpr int kMost = 16;
+    const int inner = cases[0]->inner;
     std::vector<int> lc;
     for (fvm_case* c : cases) {
-        if (!plan_coarse_levels(c, kMost, true, c->coarse_many))
-            return fail(FVM_ERR_INVALID, "batched case: no plan for its coarse levels");
-        lc.push_back(c->coarse_many.lc);
+        CoarsePlan& cp = c->coarse_many;
+        if (cluster_blocks(kMost, kMost, [&](int S) {
+                return plan_coarse_levels(c, S, true, cp) && prepare_coarse_many(inner, S, cp.smem) == cudaSuccess;
+            }) == 0)
+            return fail(FVM_ERR_CUDA, "batched case: the coarse-level kernel cannot run on this device");
+        lc.push_back(cp.lc);
     }
-    for (int S = coarse_cluster_for((int)cases.size()); S <= kMost; S *= 2) {
-        bool fits = true;
-        for (size_t i = 0; i < cases.size() && fits; ++i) {
-            fvm_case* const c = cases[i];
-            fits = coarse_plan_from(level_table(c), c->level_dir, c->inner, S, lc[i], c->coarse_many);
-            if (fits) plan_coarse_sweeps(c, c->coarse_many);
-        }
-        if (fits) return FVM_OK;
-    }
-    return fail(FVM_ERR_INVALID, "batched cases: no cluster holds their coarse levels");
+    if (cluster_blocks(coarse_cluster_for((int)cases.size()), kMost, [&](int S) {
+            size_t smem = 0;
+            for (size_t i = 0; i < cases.size(); ++i) {
+                fvm_case* const c = cases[i];
+                if (!coarse_plan_from(level_table(c), c->level_dir, c->inner, S, lc[i], c->coarse_many)) return false;
+                plan_coarse_sweeps(c, c->coarse_many);
+                smem = std::max(smem, c->coarse_many.smem);
+            }
+            return prepare_coarse_many(inner, S, smem) == cudaSuccess;
+        }) == 0)
+        return fail(FVM_ERR_CUDA, "batched cases: no cluster that this device runs holds their coarse levels");
+    return FVM_OK;
 }
 
 fvm_status build_case(const Plan& pl, fvm_case* c) {
