@@ -21,6 +21,9 @@ PROBES = {   # level 1 between what a cluster of 8 and one of 16 blocks take alo
                                                     krylov=1, smoother=1, mg_rel_tol=1e-6, max_vcycles=60),
     "room_bf16": lambda: cases.room_3d(112, 80, 48, seed=3, mg_levels=4, h=0.04, precision=cases.BF16_MIXED, krylov=1,
                                        pre_sweeps=2, post_sweeps=2, inner_cycles=2, mg_rel_tol=1e-6, max_vcycles=60),
+    # (in clusters of four blocks the right-hand side and the codes of level 1 stay in global memory)
+    "channel_bf16": lambda: cases.heated_channel_3d(128, 64, 64, mg_levels=5, precision=cases.BF16_MIXED, init_perturb=0.02,
+                                                    inner_cycles=2, mg_rel_tol=1e-6, max_vcycles=60),
     "channel_fp64": lambda: cases.heated_channel_3d(64, 32, 32, mg_levels=4, precision=cases.FP64, init_perturb=0.02,
                                                     mg_rel_tol=1e-6, max_vcycles=60),
 }
