@@ -368,6 +368,12 @@ cudaError_t launch_resid_restrict(int inner, const LevelDev& Lf, const LevelDev&
                                   void* rc, void* ec0, const SolveState* st, cudaStream_t s);
 cudaError_t launch_prolong_add(int inner, const LevelDev& Lf, const LevelDev& Lc, const void* ec, void* e,
                                const SolveState* st, cudaStream_t s);
+// bytes of neighbour codes and group flags that a pass over the level reads, for the launches' byte
+// counts (the codes of single flagged groups, at walls of boxes and outlets, are left out)
+struct CodeBytes {
+    double sweep, resid, restriction, prolong, fcg;
+};
+CodeBytes code_bytes(int inner, const LevelDev& L);
 // the cluster's share of the levels: the finest level that a cluster of S blocks takes (S smaller
 // where that leaves nothing to deal out, unless exact), the partition and the layout; first: the
 // finest level that may be among them

@@ -2222,6 +2222,14 @@ static bool v4_transfer_ok(const LevelDev& Lf) {
            (Lf.N >= (1 << 20) || g_rec);
 }
 
+CodeBytes code_bytes(int inner, const LevelDev& L) {
+    const double N = (double)L.N, codes = 2.0 * N, flags = N / 8.0, either = L.solids ? codes : flags;
+    const bool quads = inner != FVM_FP64 && L.n[0] % 4 == 0, vector = quads && (L.N >= (1 << 20) || g_rec);
+    const bool transfer = inner != FVM_FP64 && v4_transfer_ok<float>(L);
+    return {vector ? flags : codes, vector ? either : codes, transfer ? either : codes, transfer ? flags : codes,
+            quads ? either + flags : 2.0 * codes};
+}
+
 cudaError_t launch_resid_restrict(int inner, const LevelDev& Lf, const LevelDev& Lc, const void* e, const void* r,
                                   void* rc, void* ec0, const SolveState* st, cudaStream_t s) {
     cudaError_t err = cudaSuccess;

@@ -748,7 +748,7 @@ fvm_status krylov_step(fvm_case* c, int zi) {
     // BF16 levels: z and the kept direction in FP32 (z from the last sweep), r in BF16
     const bool f32 = c->inner == FVM_BF16_MIXED;
     const double sz = f32 ? 4.0 : si;
-    KLAUNCH("fcg_L0", N * (4 * sz + si + sz + 20), 2,
+    KLAUNCH("fcg_L0", N * (4 * sz + si + sz + 16) + code_bytes(c->inner, L.dev).fcg, 2,
             launch_fcg(c->inner, L.dev, f32 ? (void*)c->kz : L.e[zi], L.r, c->kdir, c->p, c->kpart, c->sst,
                        c->stream));
     return FVM_OK;
@@ -800,6 +800,7 @@ fvm_status cycle(fvm_case* c, size_t l, int& out_idx) {
     cudaStream_t s = c->stream;
     const double N = (double)L.dev.N;
     const double si = (double)elem_size(c->inner);
+    const CodeBytes cb = code_bytes(c->inner, L.dev);
     const CoarsePlan& cp = coarse_of(c);
     if (l == (size_t)cp.lc) {
         const double nco = (double)c->levels.back().dev.N;
@@ -828,32 +829,32 @@ fvm_status cycle(fvm_case* c, size_t l, int& out_idx) {
             first = 1;
         }
         for (int k = 0; k < pre; ++k) {
-            KLAUNCH(lvl_name("sweep", l), 3 * N * si + 2 * N, 1,
+            KLAUNCH(lvl_name("sweep", l), 3 * N * si + cb.sweep, 1,
                     launch_sweep(c->inner, weighted(L.dev, sweep_weight(c, L.dev, npre, first + k, false)),
                                  L.e[cur], L.r, L.e[cur ^ 1], c->sst, s));
             cur ^= 1;
         }
         const bool fuse = first_sweep_fused(c, l + 1);
         const LevelDev Lcw = weighted(Lc.dev, sweep_weight(c, Lc.dev, pre_at(c, l + 1), 0, false));
-        KLAUNCH(lvl_name("resid_restrict", l), 2 * N * si + Nc * si + 2 * N + (fuse ? Nc * (si + 2) : 0.0), 1,
+        KLAUNCH(lvl_name("resid_restrict", l), 2 * N * si + Nc * si + cb.restriction + (fuse ? Nc * (si + 2) : 0.0), 1,
                 launch_resid_restrict(c->inner, L.dev, Lcw, L.e[cur], L.r, Lc.r, fuse ? Lc.e[0] : nullptr,
                                       c->sst, s));
         int ci = 0;
         ST_TRY(cycle(c, l + 1, ci));
-        KLAUNCH(lvl_name("prolong_add", l), 2 * N * si + Nc * si + 2 * N, 1,
+        KLAUNCH(lvl_name("prolong_add", l), 2 * N * si + Nc * si + cb.prolong, 1,
                 launch_prolong_add(c->inner, L.dev, Lc.dev, Lc.e[ci], L.e[cur], c->sst, s));
         const int post = npost;
         for (int k = 0; k < post; ++k) {
             const LevelDev Lw = weighted(L.dev, sweep_weight(c, L.dev, npost, k, true));
             if (l == 0 && rep == reps - 1 && k == post - 1 && !c->desc.krylov) {
-                KLAUNCH("sweep_to_p_L0", 2 * N * si + 16 * N + 2 * N, 1,
+                KLAUNCH("sweep_to_p_L0", 2 * N * si + 16 * N + cb.sweep, 1,
                         launch_sweep_to_p(c->inner, Lw, L.e[cur], L.r, c->p, c->sst, s));
             } else if (l == 0 && rep == reps - 1 && k == post - 1 && c->kz) {
                 // BF16 levels under the flexible-CG step: the correction z in FP32
-                KLAUNCH("sweep_L0", 2 * N * si + 4 * N + 2 * N, 1,
+                KLAUNCH("sweep_L0", 2 * N * si + 4 * N + cb.sweep, 1,
                         launch_sweep_to_f32(c->inner, Lw, L.e[cur], L.r, c->kz, c->sst, s));
             } else {
-                KLAUNCH(lvl_name("sweep", l), 3 * N * si + 2 * N, 1,
+                KLAUNCH(lvl_name("sweep", l), 3 * N * si + cb.sweep, 1,
                         launch_sweep(c->inner, Lw, L.e[cur], L.r, L.e[cur ^ 1], c->sst, s));
                 cur ^= 1;
             }
@@ -867,7 +868,7 @@ fvm_status cycle(fvm_case* c, size_t l, int& out_idx) {
 // level-0 residual with the norm, the stopping rule and the first pre-sweep
 fvm_status residual0(fvm_case* c, cudaGraphConditionalHandle cond, int use_cond) {
     const double N = (double)c->cd.N;
-    KLAUNCH("resid0", N * (8 + elem_size(c->prec) + 2 * elem_size(c->inner) + 2), 1,
+    KLAUNCH("resid0", N * (8 + elem_size(c->prec) + 2 * elem_size(c->inner)) + code_bytes(c->inner, c->levels[0].dev).resid, 1,
             launch_resid0(c->inner, c->prec,
                           weighted(c->levels[0].dev, sweep_weight(c, c->levels[0].dev, pre_at(c, 0), 0, false)), c->p,
                           c->b, c->levels[0].r, c->levels[0].e[0],
