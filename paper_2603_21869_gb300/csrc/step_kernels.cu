@@ -542,7 +542,8 @@ __device__ __forceinline__ void face_flux(const CaseDev& cd, int a, const St<C>&
 
 // Each face between two fluid cells is computed once and used by both: along x by the upper cell's
 // lane, which hands its flux down by a shuffle (a warp owns 31 cells of a row, its last lane only the
-// face above them), along y by the upper row, through shared memory (a block is eight rows; the
+// face above them, or the row's last cell), along y by the upper row, through shared memory (a block is
+// eight rows; the
 // topmost computes its own upper face), along z by a march of zc planes, carried in registers.  Only
 // a face towards a boundary or a solid cell belongs to one cell, which forms its ghost.
 // FP32 is bound by the issue of the flux arithmetic and its loads, FP64 by the FP64 pipe (a 64th of
@@ -654,7 +655,9 @@ __device__ void ExplicitK<S, C, kBlend>::run(const BlockAt& at) const {
     const int i = (int)at.b.x * kCells + lane, j = (int)at.b.y * nrows + row;
     const int k0 = (int)at.b.z * zc, k1 = min(nz, k0 + zc);
     const int ic = min(i, nx - 1), jc = min(j, ny - 1);
-    const bool own = lane < kCells && i < nx && j < ny;
+    // (the last lane's upper face is not its own, unless the domain ends there)
+    const bool own = i < nx && j < ny && (lane < kCells || i == nx - 1);
+    const uint32_t missing = j < ny ? 0u : 0x1000u;   // (a whole warp's row beyond the grid: its faces are nobody's)
     const int sy = nx, sz = nx * ny;
     const C nu = prm<C>(cd.nu, cd.f.nu), dt = dt_of<C>(dt_state, 0);
     const S* const nutf = nut;
@@ -662,7 +665,7 @@ __device__ void ExplicitK<S, C, kBlend>::run(const BlockAt& at) const {
     int c = ic + sy * jc + sz * k0;
     St<C> P = load_state<S, C>(in, c);
     C nutP = nut_at(P, c);
-    uint32_t f = __ldg(cd.nbf0 + c);
+    uint32_t f = __ldg(cd.nbf0 + c) | missing;
     Face<C> zlo = {};
     if (cd.active[2] && !(f & 0x1300u)) {   // the first plane's lower face inside the grid
         const St<C> B = load_state<S, C>(in, c - sz);
@@ -672,7 +675,7 @@ __device__ void ExplicitK<S, C, kBlend>::run(const BlockAt& at) const {
         const int cn = k + 1 < nz ? c + sz : c;
         const St<C> N = load_state<S, C>(in, cn);
         const C nutN = nut_at(N, cn);
-        const uint32_t fn = __ldg(cd.nbf0 + cn);
+        const uint32_t fn = __ldg(cd.nbf0 + cn) | missing;
         const bool fluid = !(f & 0x1000u);
         C rhs[6] = {(C)0, (C)0, (C)0, (C)0, (C)0, (C)0};
         C gu[3][3] = {};
@@ -1673,13 +1676,19 @@ cudaError_t launch_destruction(int prec, const CaseDev& cd, StatePtrs in, void* 
 cudaError_t launch_explicit(int prec, const CaseDev& cd, StatePtrs in, StatePtrs out, const double* dt_state,
                             const void* nut, StatePtrs base, double wb, double ws, cudaStream_t s) {
     constexpr int kCells = ExplicitK<float, float, false>::kCells;
-    // rows per block: eight, or fewer on a single plane's worth of columns that would leave half the
-    // SMs without a block (FP64 128 x 32 x 1: 26 us with eight rows, 17.5 with two).  Always eight in
-    // a batch, whose merged launch has one block shape.
+    // rows per block: eight, or as many as there are, or fewer on a single plane's worth of columns that
+    // would leave half the SMs without a block (FP64 128 x 32 x 1: 26 us with eight rows, 17.5 with two;
+    // 512 x 1 x 256: 305 us with eight rows of which one is there, 70 with one).  Always eight in a
+    // batch, whose merged launch has one block shape.
+    // Columns: 31 cells, and one more in the last (FP32 32 x 256 x 256: 120 us in two columns of which the
+    // second has one cell, 70 in one, 83 one cell a thread).
     int rows = ExplicitK<float, float, false>::kRows;
-    auto columns = [&](int r) { return (int64_t)((cd.n[0] + kCells - 1) / kCells) * ((cd.n[1] + r - 1) / r); };
-    if (!g_rec)
+    const int xcols = cd.n[0] > 1 ? (cd.n[0] - 1 + kCells - 1) / kCells : 1;
+    auto columns = [&](int r) { return (int64_t)xcols * ((cd.n[1] + r - 1) / r); };
+    if (!g_rec) {
+        while (rows > 1 && rows / 2 >= cd.n[1]) rows /= 2;
         while (rows > 2 && columns(rows) * cd.n[2] < 76) rows /= 2;
+    }
     // planes per block: the longest march (a march loads one plane and forms one layer of faces more
     // than it owns) of at most 16 that leaves 1000 blocks, counted over a batch's cases.  FP32
     // 256 x 64 x 64: 33.7 us with 4 (1152 blocks), 36 with 8; 512 x 128 x 128: 199 / 203 / 220 us
@@ -1690,8 +1699,7 @@ cudaError_t launch_explicit(int prec, const CaseDev& cd, StatePtrs in, StatePtrs
             zc = z;
             break;
         }
-    const dim3 grid((unsigned)((cd.n[0] + kCells - 1) / kCells), (unsigned)((cd.n[1] + rows - 1) / rows),
-                    (unsigned)((cd.n[2] + zc - 1) / zc));
+    const dim3 grid((unsigned)xcols, (unsigned)((cd.n[1] + rows - 1) / rows), (unsigned)((cd.n[2] + zc - 1) / zc));
     const dim3 block(32, (unsigned)rows);
     cudaError_t err = cudaSuccess;
     if (base.f[0])
