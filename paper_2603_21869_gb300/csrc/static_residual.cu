@@ -27,10 +27,11 @@ static __device__ __align__(256) double g_residual_scratch[kScratchDoubles];
 // a warp reduction of r^2 and b^2 took about 37 FP64 operations a cell, 194 us at 201 x 130 x 97
 // cells.  Now each difference across a face is formed once and used by both cells: along x by the
 // lane of the upper cell (a shuffle hands it down; 31 cells a warp), along y by a thread that owns
-// kRows rows, along z by the march, and the squares are summed in registers: 13 FP64 instructions a
-// row of 31 cells, 90 us (ncu; the pipe 75 % busy, 58 us at its rate), 95 us a call for 207.
-// A warp's item is 31 x kRows x zc cells; the items go round the warps of at most kBlocks blocks.
-constexpr int kWarps = 8, kRows = 4, kLanes = 31;
+// kRows (4) rows, along z by the march, and the squares are summed in registers: 13 FP64 instructions a
+// row of 31 cells, 81 us a call for 194 (58 us at the pipe's rate).
+// A warp's item is 31 x kRows x zc cells; the items go round the warps of at most kBlocks blocks, or one to
+// a block first where there are few.
+constexpr int kWarps = 8, kLanes = 31;
 constexpr int kBlocks = 304;                            // two blocks on each of 152 SMs
 
 struct Tiles {
@@ -39,11 +40,12 @@ struct Tiles {
 
 // r = b - A p on a box without obstacles: a face of the domain is
 // zero-gradient (dirichlet[face] = 0) or zero-value (1) for p.
+template <int kRows>
 __global__ void __launch_bounds__(32 * kWarps) k_residual_static(const double* __restrict__ p,
                                                                  const double* __restrict__ b, double* __restrict__ r,
                                                                  double* __restrict__ norms, double* scratch, int nx,
                                                                  int ny, int nz, double ih2x, double ih2y, double ih2z,
-                                                                 unsigned dir_mask, Tiles tiles) {
+                                                                 unsigned dir_mask, Tiles tiles, int few) {
     __shared__ double red[2][kWarps];
     __shared__ bool last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -54,7 +56,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_residual_static(const double* _
     };
     double r2 = 0.0, b2 = 0.0;
     const int total = tiles.x * tiles.y * tiles.z;
-    for (int t = blockIdx.x * kWarps + warp; t < total; t += gridDim.x * kWarps) {
+    for (int t = few ? warp * gridDim.x + blockIdx.x : blockIdx.x * kWarps + warp; t < total; t += gridDim.x * kWarps) {
         const int tx = t % tiles.x, ty = (t / tiles.x) % tiles.y, tz = t / (tiles.x * tiles.y);
         // lane l holds cell i: the warp's cells and the one after them (at the top face its ghost)
         const int i = tx * kLanes + lane, j0 = ty * kRows;
@@ -66,44 +68,61 @@ __global__ void __launch_bounds__(32 * kWarps) k_residual_static(const double* _
             const double v = __ldg(p + ic + sy * min(max(j, 0), ny - 1) + sz * k);
             return i >= nx ? ghost(1, v) : v;
         };
+        // what plane k needs beside plane k itself, asked for a plane ahead (the item's first plane
+        // together with planes k0 and k0 - 1: a small grid's call is one round trip to memory; 33 x 33 x 33
+        // cells 14.0 -> 12.4 us, 201 x 130 x 97 83 -> 81)
+        double pn[kRows], bv[kRows], edge[kRows], below, above;
+        auto fetch = [&](int k) {
+#pragma unroll
+            for (int q = 0; q < kRows; ++q) {
+                const int c = ic + sy * min(j0 + q, ny - 1) + sz * k;
+                pn[q] = at(j0 + q, min(k + 1, nz - 1));
+                bv[q] = __ldg(b + c);
+                edge[q] = lane == 0 && i > 0 ? __ldg(p + c - 1) : 0.0;
+            }
+            below = at(j0 - 1, k);            // (clamped: at the faces not used)
+            above = at(j0 + kRows, k);
+        };
         double pc[kRows], dz[kRows];   // plane k, and its difference to plane k - 1
 #pragma unroll
         for (int q = 0; q < kRows; ++q) {
             pc[q] = at(j0 + q, k0);
-            dz[q] = pc[q] - (k0 > 0 ? at(j0 + q, k0 - 1) : ghost(4, pc[q]));
+            dz[q] = at(j0 + q, max(k0 - 1, 0));
         }
+        fetch(k0);
+#pragma unroll
+        for (int q = 0; q < kRows; ++q) dz[q] = pc[q] - (k0 > 0 ? dz[q] : ghost(4, pc[q]));
         for (int k = k0; k < k1; ++k) {
-            double pn[kRows], bv[kRows], xm[kRows];
+            double xm[kRows], up[kRows], bk[kRows];
 #pragma unroll
             for (int q = 0; q < kRows; ++q) {
-                pn[q] = k + 1 < nz ? at(j0 + q, k + 1) : ghost(5, pc[q]);
-                const int c = ic + sy * min(j0 + q, ny - 1) + sz * k;
-                bv[q] = __ldg(b + c);
+                up[q] = k + 1 < nz ? pn[q] : ghost(5, pc[q]);
+                bk[q] = bv[q];
                 xm[q] = __shfl_up_sync(0xffffffffu, pc[q], 1);
-                if (lane == 0) xm[q] = i > 0 ? __ldg(p + c - 1) : ghost(0, pc[q]);
+                if (lane == 0) xm[q] = i > 0 ? edge[q] : ghost(0, pc[q]);
             }
-            const double below = j0 > 0 ? at(j0 - 1, k) : ghost(2, pc[0]);
-            const double above = j0 + kRows < ny ? at(j0 + kRows, k) : 0.0;   // (the last row's ghost: below)
-            double dy = pc[0] - below;
+            const double lo = j0 > 0 ? below : ghost(2, pc[0]), hi4 = above;
+            if (k + 1 < k1) fetch(k + 1);
+            double dy = pc[0] - lo;
 #pragma unroll
             for (int q = 0; q < kRows; ++q) {
                 const double dx = pc[q] - xm[q];                          // i > 0 .. nx: to the cell below
                 const double dxu = __shfl_down_sync(0xffffffffu, dx, 1);  // its other face
-                const double hi = j0 + q + 1 >= ny ? ghost(3, pc[q]) : (q + 1 < kRows ? pc[q + 1 < kRows ? q + 1 : q] : above);
-                const double dyu = hi - pc[q], dzu = pn[q] - pc[q];
+                const double hi = j0 + q + 1 >= ny ? ghost(3, pc[q]) : (q + 1 < kRows ? pc[q + 1 < kRows ? q + 1 : q] : hi4);
+                const double dyu = hi - pc[q], dzu = up[q] - pc[q];
                 double Ap = 0.0;
                 if (nx > 1) Ap += (dx - dxu) * ih2x;
                 if (ny > 1) Ap += (dy - dyu) * ih2y;
                 if (nz > 1) Ap += (dz[q] - dzu) * ih2z;
-                const double rv = bv[q] - Ap;
+                const double rv = bk[q] - Ap;
                 if (own && q < rows) {
                     r[i + sy * (j0 + q) + sz * k] = rv;
                     r2 = fma(rv, rv, r2);
-                    b2 = fma(bv[q], bv[q], b2);
+                    b2 = fma(bk[q], bk[q], b2);
                 }
                 dy = dyu;
                 dz[q] = dzu;
-                pc[q] = pn[q];
+                pc[q] = up[q];
             }
         }
     }
@@ -207,16 +226,34 @@ extern "C" fvm_status fvm_poisson_residual_static(const double* p, const double*
                        "65,535 along y and z)");
         return FVM_ERR_INVALID;
     }
+    // the axes with more than one cell, in their order (a collapsed one changes no index): rows and planes
+    // of a warp's item are then there (200 x 1 x 200 cells: 26 us with three of four rows missing, 12.4 so)
+    int n[3] = {1, 1, 1}, axes = 0;
+    double ih2[3] = {0.0, 0.0, 0.0};
+    unsigned mask = 0;
+    const int given[3] = {nx, ny, nz};
+    for (int a = 0; a < 3; ++a) {
+        if (given[a] == 1) continue;
+        n[axes] = given[a];
+        ih2[axes] = 1.0 / (h[a] * h[a]);
+        for (int side = 0; side < 2; ++side)
+            if (dirichlet[2 * a + side]) mask |= 1u << (2 * axes + side);
+        ++axes;
+    }
+    // rows per item: four, or one where items of four rows and one plane are fewer than blocks (a chain of
+    // four rows takes longer than the launch: 31 x 31 x 31 cells 27.5 us at four rows and planes, 10.7 so,
+    // as one cell a thread)
+    Tiles tiles;
+    tiles.x = (int)(((int64_t)n[0] + kLanes - 1) / kLanes);
+    const int rows = (int64_t)tiles.x * (((int64_t)n[1] + 3) / 4) * n[2] <= kBlocks ? 1 : 4;
+    tiles.y = (int)(((int64_t)n[1] + rows - 1) / rows);
     // planes per item: the fewest rounds of items over the 608 warp schedulers times the planes of a
     // round (one more for the difference an item starts with), and three rounds or more where the
     // grid has them (two warps a scheduler kept the FP64 pipe only two thirds busy)
-    Tiles tiles;
-    tiles.x = (int)(((int64_t)nx + kLanes - 1) / kLanes);
-    tiles.y = (int)(((int64_t)ny + kRows - 1) / kRows);
     int64_t best = 0, tiles_rounds = 0;
-    for (int zc = 32; zc >= 4; --zc) {
-        const int64_t z = ((int64_t)nz + zc - 1) / zc, rounds = ((int64_t)tiles.x * tiles.y * z + 607) / 608;
-        const int64_t cost = rounds * ((nz < zc ? nz : zc) + 1);
+    for (int zc = 32; zc >= 1; --zc) {
+        const int64_t z = ((int64_t)n[2] + zc - 1) / zc, rounds = ((int64_t)tiles.x * tiles.y * z + 607) / 608;
+        const int64_t cost = rounds * ((n[2] < zc ? n[2] : zc) + 1);
         if (best == 0 || tiles_rounds < 3 || (cost < best && rounds >= 3)) {
             best = cost;
             tiles_rounds = rounds;
@@ -224,9 +261,12 @@ extern "C" fvm_status fvm_poisson_residual_static(const double* p, const double*
             tiles.zc = zc;
         }
     }
-    const int64_t total = ((int64_t)tiles.x * tiles.y * tiles.z + kWarps - 1) / kWarps;   // (items below 2^20)
+    // few: up to four warps' items a block, dealt out over the blocks first
+    const int64_t total = (int64_t)tiles.x * tiles.y * tiles.z;   // (below 2^20)
+    const bool few = total <= 4 * kBlocks;
+    const int64_t blocks = few ? total : (total + kWarps - 1) / kWarps;
     const dim3 block(32 * kWarps);
-    const dim3 grid((unsigned)(total < kBlocks ? total : kBlocks));
+    const dim3 grid((unsigned)(blocks < kBlocks ? blocks : kBlocks));
     double* scratch = nullptr;
     std::string err;
     fvm_status st = scratch_for_current_device(&scratch, err);
@@ -234,15 +274,12 @@ extern "C" fvm_status fvm_poisson_residual_static(const double* p, const double*
         set_last_error(err);
         return st;
     }
-    unsigned mask = 0;
-    for (int f = 0; f < 6; ++f)
-        if (dirichlet[f]) mask |= 1u << f;
     cudaStream_t s = (cudaStream_t)stream;
     // the block counter must start at zero (a memset, not an allocation)
     cudaError_t e = cudaMemsetAsync(scratch + 2 * kMaxBlocks, 0, sizeof(unsigned), s);
     if (e == cudaSuccess) {
-        k_residual_static<<<grid, block, 0, s>>>(p, b, r, norms, scratch, nx, ny, nz, 1.0 / (h[0] * h[0]),
-                                                 1.0 / (h[1] * h[1]), 1.0 / (h[2] * h[2]), mask, tiles);
+        const auto kernel = rows == 1 ? k_residual_static<1> : k_residual_static<4>;
+        kernel<<<grid, block, 0, s>>>(p, b, r, norms, scratch, n[0], n[1], n[2], ih2[0], ih2[1], ih2[2], mask, tiles, few);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) {
