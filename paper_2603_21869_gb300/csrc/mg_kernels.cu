@@ -913,9 +913,9 @@ __device__ __forceinline__ void fcg_reduce(T (&s)[4], double* partials, SolveSta
 }
 
 // ------------------------------------------------------------------ level 0 residual in float-float
-// The reduced-precision cases hold p as double-float pairs (pp_load); this
-// path evaluates r = b - A p without the FP64 pipe (1/64 of the FP32 rate
-// here): the stencil runs in double-float arithmetic (Dekker's error-free sum
+// The reduced-precision cases hold p as double-float pairs (pp_load); on large
+// levels and in batches this path evaluates r = b - A p without the FP64 pipe
+// (1/64 of the FP32 rate here): the stencil runs in double-float arithmetic (Dekker's error-free sum
 // and FMA-based product), about 2^-48 relative accuracy.  As a difference
 // form, A p = sum_a ih2_a ((P - g_lo) + (P - g_hi)) with g the neighbour
 // (code 0), P (zero-gradient: no term) or -P (zero-value: 2P), which equals

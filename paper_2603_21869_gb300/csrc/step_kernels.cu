@@ -542,10 +542,9 @@ __device__ __forceinline__ void face_flux(const CaseDev& cd, int a, const St<C>&
 
 // Each face between two fluid cells is computed once and used by both: along x by the upper cell's
 // lane, which hands its flux down by a shuffle (a warp owns 31 cells of a row, its last lane only the
-// face above them, or the row's last cell), along y by the upper row, through shared memory (a block is
-// eight rows; the
-// topmost computes its own upper face), along z by a march of zc planes, carried in registers.  Only
-// a face towards a boundary or a solid cell belongs to one cell, which forms its ghost.
+// face above them, or the row's last cell), along y by the upper row, through shared memory (a block
+// is eight rows; the topmost computes its own upper face), along z by a march of zc planes, carried in
+// registers.  Only a face towards a boundary or a solid cell belongs to one cell, which forms its ghost.
 // FP32 is bound by the issue of the flux arithmetic and its loads, FP64 by the FP64 pipe (a 64th of
 // the FP32 rate); a thread a cell computed every inner face twice.  One cell a thread -> this, us a
 // launch: FP32 256 x 64 x 64 36.8 -> 33.7, 512 x 128 x 128 266 -> 203, BF16-mixed room
