@@ -1487,21 +1487,27 @@ struct FcgUpdVK {
                 if (!is_solid(fs[t])) u[t] = fma(alpha, d[t], u[t]);
             VecW<double, W>::store(p, c, u);
         } else {
-            float step[W];
+            float wide[W];   // alpha d where it is formed in a wider type (else at its use: one multiply-add)
+            if constexpr (sizeof(T) > sizeof(C)) {
 #pragma unroll
-            for (int t = 0; t < W; ++t) d[t] *= alpha;
-            narrowed(d, step);
+                for (int t = 0; t < W; ++t) d[t] *= alpha;
+                narrowed(d, wide);
+            }
+            auto step = [&](int t) -> float {
+                if constexpr (sizeof(T) > sizeof(C)) return wide[t];
+                else return alpha * d[t];
+            };
             float4* pp = reinterpret_cast<float4*>(p + c);   // p as double-float pairs, two cells per 16 bytes
 #pragma unroll
             for (int h = 0; h < W / 2; ++h) {
                 float4 u = pp[h];
                 if (!codes || !is_solid(fs[2 * h])) {
-                    const float2 x = pp_plus(make_float2(u.x, u.y), step[2 * h]);
+                    const float2 x = pp_plus(make_float2(u.x, u.y), step(2 * h));
                     u.x = x.x;
                     u.y = x.y;
                 }
                 if (!codes || !is_solid(fs[2 * h + 1])) {
-                    const float2 x = pp_plus(make_float2(u.z, u.w), step[2 * h + 1]);
+                    const float2 x = pp_plus(make_float2(u.z, u.w), step(2 * h + 1));
                     u.z = x.x;
                     u.w = x.y;
                 }
